@@ -453,7 +453,7 @@ cudaError_t cum_factor_in(Handle& h, unsigned long long* counters, cudaStream_t 
     for (int k0 = 0; k0 < ns; k0 += kCumPanel) {
       const int kb = std::min(kCumPanel, ns - k0);
       const int kd = kt_begin(h, kFamDiag, (2.0 / 3.0) * kb * kb * kb, st);
-      k_dense_diag_t<T><<<1, 256, 0, st>>>(Q, n2, k0, kb, 0, PivotRule{}, counters);
+      launch_dense_diag<T>(Q, n2, k0, kb, 1, 0, PivotRule{}, counters, st);
       kt_end(h, kd, st);
       h.launches++;
       const int rest = rend - k0 - kb;

@@ -31,43 +31,92 @@ struct PivotRule {
   const int32_t* primal = nullptr; // per column of the matrix: 1 if primal
 };
 
-// Pairs (i, j) with 1 <= j <= i < 64 ordered by j descending, then i: the
-// pairs with j >= r0 are the first (64 - r0)(65 - r0) / 2 entries, so a
-// trailing triangle of the diagonal block spreads evenly over the threads.
-constexpr int kDiagPairs = (kPanelW - 1) * kPanelW / 2;
+// LDL^T of the diagonal block at (k0, k0) of matrix blockIdx.x, in shared
+// memory, in sub-panels of kSub = 8 columns:
+//   (1) the sub-panel with all its rows, right-looking, by four warps (one per
+//       SM sub-partition) that hold it in registers: a lane per row, the
+//       columns dealt out over the warps (two warps per column set while more
+//       than 32 rows are left, four sets of columns afterwards).  One barrier
+//       per pivot: the warps that own the pivot's column publish it in shared
+//       memory, every thread forms the same 1 / d and its own l = u / d, and the
+//       next pivot's column is updated and published first;
+//   (2) the trailing triangle of the block takes A[i][j] -= sum_c L[i][c] U[j][c]
+//       over the sub-panel, spread over all threads (rows p and R-1-p of the
+//       triangle of order R together hold R + 1 entries).
+// What bounds it: FP64 on one SM.  An FP64 operation keeps its sub-partition's
+// pipe busy for 64 cycles per warp, so the chain of a pivot (the reciprocal,
+// l, the next column's entry, a barrier: about 540 cycles) and the 64^3 / 6
+// multiply-adds of the block both count.  Sub-panels of 8 keep few of those in
+// the chain's steps; 16 took 10% longer.  64 FP64 pivots of one matrix take
+// 31 us (69 with a barrier pair per pivot, the reciprocal on one thread and a
+// thread per row below a sub-panel's diagonal block), 32 pivots 9.6 us (26.8);
+// FP32, where only barriers and shared memory count, 10.8 us per 64 (24.5).
+constexpr int kSub = 8;
 
-__device__ __forceinline__ void diag_pair(int p, int& i, int& j) {
-  // group t = 64 - j holds pairs [t(t-1)/2, t(t+1)/2)
-  int t = (int)((sqrtf(8.0f * p + 1.0f) + 1.0f) * 0.5f);
-  while (t * (t - 1) / 2 > p) t--;
-  while (t * (t + 1) / 2 <= p) t++;
-  j = kPanelW - t;
-  i = j + (p - t * (t - 1) / 2);
+__device__ __forceinline__ void bar_sync_warps03() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+
+// Phase (1) for the thread that holds row `row` and the columns q G + g of the
+// sub-panel at column c0 (cb <= 16 pivots).  Entries above the diagonal and
+// rows past the block are carried along and never stored.
+// RULE: the pivot rule applies; repl holds the replacement of each of the
+// block's pivots, +-thr, and thr's bit pattern is compared with the pivot's
+// (non-negative doubles order like their bits, and a comparison of integers
+// leaves the FP64 pipe alone).  There are no branches around the multiply-adds:
+// a column that is done takes the last one or two updates of its set along,
+// unused.
+template <class T, int G, bool RULE>
+__device__ __forceinline__ int diag_subpanel(T (&A)[kPanelW][kPanelW + 1], T (&U)[kPanelW][kSub + 1],
+                                             T (&col)[2][kPanelW], const T* repl, int c0, int cb, int row, int g) {
+  constexpr int NQ = kSub / G;
+  int pert = 0;
+  T a[NQ];
+#pragma unroll
+  for (int q = 0; q < NQ; q++) a[q] = A[row][c0 + q * G + g];
+  if (g == 0) col[0][row] = a[0];
+  bar_sync_warps03();
+#pragma unroll
+  for (int k = 0; k < kSub; k++) {
+    if (k < cb) {
+      const T* ck = col[k & 1];
+      const T u = ck[row];
+      T d = ck[c0 + k];
+      T uj[NQ];  // all loads first
+#pragma unroll
+      for (int q = (k + 1) / G; q < NQ; q++) uj[q] = ck[c0 + q * G + g];
+      if constexpr (RULE) {
+        const T t = repl[c0 + k];
+        const long long mag = 0x7fffffffffffffffLL;
+        const bool small = (__double_as_longlong((double)d) & mag) < (__double_as_longlong((double)t) & mag);
+        d = small ? t : d;
+        pert += small;
+      }
+      const T l = u * pivot_recip(d);
+#pragma unroll
+      for (int q = (k + 1) / G; q < NQ; q++) {
+        a[q] -= l * uj[q];
+        // the next pivot's column is published as soon as it is updated
+        if (q == (k + 1) / G && g == (k + 1) % G) col[(k + 1) & 1][row] = a[q];
+      }
+      if (g == k % G) {  // (above the diagonal: unused entries)
+        U[row][k] = u;
+        A[row][c0 + k] = row == c0 + k ? d : l;
+      }
+      bar_sync_warps03();
+    }
+  }
+  return pert;
 }
 
-// LDL^T of the diagonal block at (k0, k0) of matrix blockIdx.x, in shared
-// memory, in sub-panels of kSub = 16 columns:
-//   (1) the 16 x 16 diagonal sub-block, one thread per entry, a barrier pair
-//       per column (thread 0 applies the pivot rule and forms 1/d; the
-//       trailing entries take -l_i u_j; the column is scaled one step late,
-//       after its unscaled values have been used);
-//   (2) the rows below it in the block solve y L11^T = a, one thread per row
-//       (Y = y kept unscaled, L = y D^{-1});
-//   (3) the trailing triangle of the block takes A[i][j] -= sum_c L[i][c] Y[j][c]
-//       over the sub-panel, spread over all threads through the pair table.
-constexpr int kSub = 16;
-
-template <class T>
+template <class T, bool RULE>
 __global__ void __launch_bounds__(256, 1) k_dense_diag_t(T* __restrict__ S0, int n, int k0, int kb,
                                                       int64_t bstride, PivotRule rule,
                                                       unsigned long long* __restrict__ counters) {
   __shared__ T A[kPanelW][kPanelW + 1];
-  __shared__ T Ys[kPanelW][kSub + 1];
-  __shared__ T Dinv[kSub];
-  __shared__ uint16_t pairs[kDiagPairs];
-  __shared__ int pert;
+  __shared__ T U[kPanelW][kSub + 1];
+  __shared__ T col[2][kPanelW];
+  __shared__ T repl[RULE ? kPanelW : 1];
   T* S = S0 + (int64_t)blockIdx.x * bstride;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   {
     // 16 loads per thread issued together, then stored
     T v[16];
@@ -76,75 +125,40 @@ __global__ void __launch_bounds__(256, 1) k_dense_diag_t(T* __restrict__ S0, int
       const int q = tid + u * 256, c = q >> 6, r = q & 63;
       v[u] = (r >= c && r < kb && c < kb) ? S[(int64_t)(k0 + r) + (int64_t)(k0 + c) * n] : T(0);
     }
+    if (RULE && tid < kb) {
+      // a threshold that is not positive (or NaN) leaves every pivot alone
+      const double thr = rule.pivot_eps * rule.anorm[blockIdx.x];
+      repl[tid] = thr > 0.0 ? (T)(rule.primal[k0 + tid] ? thr : -thr) : T(0);
+    }
 #pragma unroll
     for (int u = 0; u < 16; u++) {
       const int q = tid + u * 256, c = q >> 6, r = q & 63;
       A[r][c] = v[u];
     }
   }
-  for (int p = tid; p < kDiagPairs; p += blockDim.x) {
-    int i, j;
-    diag_pair(p, i, j);
-    pairs[p] = (uint16_t)(i | (j << 8));
-  }
-  if (tid == 0) pert = 0;
+  int pert = 0;
   __syncthreads();
-  const double thr = rule.anorm ? rule.pivot_eps * rule.anorm[blockIdx.x] : 0.0;
-  const int si = tid >> 4, sj = tid & 15;  // this thread's entry of a 16 x 16 sub-block
   for (int c0 = 0; c0 < kb; c0 += kSub) {
     const int cb = min(kSub, kb - c0);
-    for (int c = 0; c < cb; c++) {  // (1)
-      if (tid == 0) {
-        T d = A[c0 + c][c0 + c];
-        if (thr > 0.0 && fabs((double)d) < thr) {
-          d = (T)(rule.primal[k0 + c0 + c] ? thr : -thr);
-          A[c0 + c][c0 + c] = d;
-          pert++;
-        }
-        Dinv[c] = pivot_recip(d);
+    if (warp < 4) {  // (1)
+      if (kb > 32 && c0 < 32)
+        pert += diag_subpanel<T, 2, RULE>(A, U, col, repl, c0, cb, (warp & 1) * 32 + lane, warp >> 1);
+      else
+        pert += diag_subpanel<T, 4, RULE>(A, U, col, repl, c0, cb, (c0 & 32) + lane, warp);
+    }
+    __syncthreads();
+    const int r0 = c0 + cb, R = kb - r0;
+    if (R > 0) {  // (2) (only the last sub-panel is ragged: cb == kSub here)
+      for (int q = tid; q < R * (R + 1) / 2; q += 256) {
+        const int p = q / (R + 1), off = q - p * (R + 1);
+        const int i = off < R - p ? R - 1 - p : p, j = off < R - p ? off : off - (R - p);
+        T acc = T(0);
+#pragma unroll
+        for (int c = 0; c < kSub; c++) acc += A[r0 + i][c0 + c] * U[r0 + j][c];
+        A[r0 + i][r0 + j] -= acc;
       }
-      if (c > 0 && sj == c - 1 && si > c - 1 && si < cb) A[c0 + si][c0 + c - 1] *= Dinv[c - 1];
       __syncthreads();
-      if (si > c && sj > c && sj <= si && si < cb)
-        A[c0 + si][c0 + sj] -= A[c0 + si][c0 + c] * Dinv[c] * A[c0 + sj][c0 + c];
-      __syncthreads();
     }
-    if (sj == cb - 1 && si > cb - 1 && si < cb) A[c0 + si][c0 + cb - 1] *= Dinv[cb - 1];
-    __syncthreads();
-    const int r0 = c0 + cb;
-    for (int row = r0 + tid; row < kb; row += blockDim.x) {  // (2)
-      T y[kSub];
-#pragma unroll
-      for (int c = 0; c < kSub; c++) {
-        if (c < cb) {
-          T acc = A[row][c0 + c];
-#pragma unroll
-          for (int c2 = 0; c2 < c; c2++) acc -= y[c2] * A[c0 + c][c0 + c2];
-          y[c] = acc;
-        }
-      }
-#pragma unroll
-      for (int c = 0; c < kSub; c++)
-        if (c < cb) {
-          Ys[row][c] = y[c];
-          A[row][c0 + c] = y[c] * Dinv[c];
-        }
-    }
-    __syncthreads();
-    if (r0 < kb) {  // (3): pairs with j >= r0
-      const int npairs = (kPanelW - r0) * (kPanelW - r0 + 1) / 2;
-      for (int p = tid; p < npairs; p += blockDim.x) {
-        const int ij = pairs[p], i = ij & 0xFF, j = ij >> 8;
-        if (i < kb) {
-          T acc = T(0);
-#pragma unroll
-          for (int c = 0; c < kSub; c++)
-            if (c < cb) acc += A[i][c0 + c] * Ys[j][c];
-          A[i][j] -= acc;
-        }
-      }
-    }
-    __syncthreads();
   }
   {
 #pragma unroll
@@ -302,6 +316,14 @@ inline cudaError_t launch_prio(void (*kernel)(KArgs...), dim3 grid, dim3 block, 
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+// The diagonal block of nb matrices (with the pivot rule if it is on).
+template <class T>
+inline void launch_dense_diag(T* S, int n, int k0, int kb, int nb, int64_t bstride, const PivotRule& rule,
+                              unsigned long long* counters, cudaStream_t st, int prio = 0) {
+  launch_prio(rule.anorm ? k_dense_diag_t<T, true> : k_dense_diag_t<T, false>, dim3(nb), dim3(256), 0, st, prio, S, n,
+              k0, kb, bstride, rule, counters);
 }
 
 // Rows below the diagonal block of nb matrices.  A thread per row issues the

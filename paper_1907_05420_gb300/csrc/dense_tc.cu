@@ -1522,7 +1522,7 @@ cudaError_t factor_tc(Handle& h, T* S, T* Y, int n, int npiv, int nb, const TcSt
   for (int k0 = 0; k0 < npiv && e == cudaSuccess; k0 += TK) {
     const int kb = std::min(TK, npiv - k0);
     const int kd = kt_begin(h, kFamDiag, nb * (2.0 / 3.0) * kb * kb * kb, st);
-    launch_prio(k_dense_diag_t<T>, dim3(nb), dim3(256), 0, st, prio, S, n, k0, kb, ts.s, rule, counters);
+    launch_dense_diag<T>(S, n, k0, kb, nb, ts.s, rule, counters, st, prio);
     kt_end(h, kd, st);
     h.launches++;
     // rows below the envelope of the panel's columns stay zero (no pivoting)
@@ -1642,7 +1642,7 @@ cudaError_t factor_emu_wide(Handle& h, double* S, int n, int npiv, int nb, const
     for (int c = 0; c * TK < Wb && e == cudaSuccess; c++) {
       const int k0 = K0 + c * TK, kb = std::min(TK, npiv - k0);
       const int kd = kt_begin(h, kFamDiag, nb * (2.0 / 3.0) * kb * kb * kb, st);
-      launch_prio(k_dense_diag_t<double>, dim3(nb), dim3(256), 0, st, prio, S, n, k0, kb, ts.s, rule, counters);
+      launch_dense_diag<double>(S, n, k0, kb, nb, ts.s, rule, counters, st, prio);
       kt_end(h, kd, st);
       h.launches++;
       const int m = n - k0 - kb;
@@ -1756,8 +1756,7 @@ cudaError_t factor_tf32_wide(Handle& h, float* S, float* Y, int n, unsigned long
     for (int c = 0; c * TK < Wb && e == cudaSuccess; c++) {
       const int k0 = K0 + c * TK, kb = std::min(TK, n - k0);
       const int kd = kt_begin(h, kFamDiag, (2.0 / 3.0) * kb * kb * kb, st);
-      launch_prio(k_dense_diag_t<float>, dim3(1), dim3(256), 0, st, prio, S, n, k0, kb, (int64_t)0, PivotRule{},
-                  counters);
+      launch_dense_diag<float>(S, n, k0, kb, 1, 0, PivotRule{}, counters, st, prio);
       kt_end(h, kd, st);
       h.launches++;
       const int m = n - k0 - kb;
@@ -1946,7 +1945,7 @@ cudaError_t launch_dense_diag_panel_f64(Handle& h, int k0, int kb, int rend, uns
                                         cudaStream_t st) {
   const int n = h.nC;
   const int kd = kt_begin(h, kFamDiag, (2.0 / 3.0) * kb * kb * kb, st);
-  k_dense_diag_t<double><<<1, 256, 0, st>>>(h.S, n, k0, kb, 0, PivotRule{}, counters);
+  launch_dense_diag<double>(h.S, n, k0, kb, 1, 0, PivotRule{}, counters, st);
   kt_end(h, kd, st);
   h.launches++;
   if (rend - k0 - kb > 0) {

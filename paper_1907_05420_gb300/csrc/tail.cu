@@ -237,7 +237,7 @@ cudaError_t launch_dense_tail(Handle& h, cudaStream_t st) {
   for (int k0 = 0; h.tail_mode == 1 && k0 < nT; k0 += kPanelW) {
     const int kb = std::min(kPanelW, nT - k0);
     const int kd = kt_begin(h, kFamDiag, N * (2.0 / 3.0) * kb * kb * kb, st);
-    k_dense_diag_t<double><<<N, 256, 0, st>>>(h.Tt, nTa, k0, kb, t2, rule, h.counters);
+    launch_dense_diag<double>(h.Tt, nTa, k0, kb, N, t2, rule, h.counters, st);
     kt_end(h, kd, st);
     h.launches++;
     const int rest = nTa - k0 - kb;

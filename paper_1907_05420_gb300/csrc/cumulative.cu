@@ -149,37 +149,7 @@ __global__ void k_cum_build(const double* __restrict__ Sd, const double* __restr
   }
 }
 
-// Trailing update of one period's partial factor, A[i][j] -= sum_c Y[i][c]
-// L[j][c] for base <= j <= i < rend: a 16 x 16 tile of the lower triangle per
-// CTA, one entry per thread.  The trailing matrices here are small (2 n_s
-// rows), so small tiles spread each update over many SMs.
-constexpr int kCumTile = 16;
 constexpr int kCumPanel = 32;  // pivot columns per panel of the period factors
-
-template <class T>
-__global__ void __launch_bounds__(kCumTile * kCumTile) k_cum_update(T* __restrict__ S, const T* __restrict__ Y, int n,
-                                                                   int k0, int kb, int rend) {
-  const int base = k0 + kb;
-  int tile = blockIdx.x, ti = 0;
-  while (tile > ti) {
-    tile -= ti + 1;
-    ti++;
-  }
-  const int i0 = base + ti * kCumTile, j0 = base + tile * kCumTile;
-  __shared__ T Ys[kCumPanel][kCumTile + 1];
-  __shared__ T Ls[kCumPanel][kCumTile + 1];
-  const int tx = threadIdx.x % kCumTile, ty = threadIdx.x / kCumTile;
-  for (int q = threadIdx.x; q < kb * kCumTile; q += blockDim.x) {
-    const int c = q / kCumTile, r = q % kCumTile;
-    Ys[c][r] = i0 + r < rend ? Y[(i0 + r) + (int64_t)c * n] : T(0);
-    Ls[c][r] = j0 + r < rend ? S[(j0 + r) + (int64_t)(k0 + c) * n] : T(0);
-  }
-  __syncthreads();
-  T acc = T(0);
-  for (int c = 0; c < kb; c++) acc += Ys[c][ty] * Ls[c][tx];
-  const int i = i0 + ty, j = j0 + tx;
-  if (i < rend && j <= i) S[i + (int64_t)j * n] -= acc;
-}
 
 // Z L_j = [I; L21_j] for the rows of Z: rows < ns give Linv_j = L_j^{-1}, the
 // others M_j = L21_j L_j^{-1} (stored also transposed); D_j is copied out.
@@ -459,9 +429,8 @@ cudaError_t cum_factor_in(Handle& h, unsigned long long* counters, cudaStream_t 
       const int rest = rend - k0 - kb;
       if (rest > 0) {
         launch_dense_panel<T>(Q, QY, n2, k0, kb, rend, 1, 0, 0, st);
-        const int tiles = (rest + kCumTile - 1) / kCumTile;
         const int kt = kt_begin(h, kFamDenseF64, update_flops(rest, 0, rest, kb), st);
-        k_cum_update<T><<<tiles * (tiles + 1) / 2, kCumTile * kCumTile, 0, st>>>(Q, QY, n2, k0, kb, rend);
+        launch_dense_update<T>(Q, QY, n2, k0, kb, rend, 1, 0, 0, st);
         kt_end(h, kt, st);
         h.launches += 2;
       }

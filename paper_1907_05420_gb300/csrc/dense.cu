@@ -7,7 +7,7 @@
 //   panel: L21 = A21 L11^{-T} D1^{-1}, Y = L21 D1 kept for the update
 //     (k_dense_diag_t / k_dense_panel_t in dense_kernels.cuh, shared with the
 //     tensor-core modes and the dense tail of the block factors);
-//   k_dense_update: A22 -= Y L21^T on the lower-triangle 64 x 64 tiles (FP64).
+//   k_dense_update: A22 -= Y L21^T on the lower-triangle 16 x 16 tiles (FP64).
 // No pivoting: S is positive definite when the blocks are quasidefinite and C
 // is positive definite; a zero pivot is counted and reported.
 #include "dense_kernels.cuh"
@@ -294,9 +294,8 @@ cudaError_t launch_dense_ldlt(Handle& h, unsigned long long* counters, cudaStrea
     if (e != cudaSuccess) return e;
     const int rest = rend - k0 - kb;
     if (rest > 0) {
-      const int T = (rest + 63) / 64;
       const int kt = kt_begin(h, kFamDenseF64, update_flops(rest, 0, rest, kb), st);
-      k_dense_update<<<T * (T + 1) / 2, 256, 0, st>>>(h.S, h.Ypanel, n, k0, kb, rend, 0, 0);
+      launch_dense_update<double>(h.S, h.Ypanel, n, k0, kb, rend, 1, 0, 0, st);
       kt_end(h, kt, st);
       h.launches++;
     }

@@ -8,7 +8,7 @@
 // Per panel:
 //   k_dense_diag_t:   LDL^T of the kb x kb diagonal block;
 //   k_dense_panel_t:  L21 = A21 L11^{-T} D1^{-1} and Y = L21 D1 (rows below);
-//   k_dense_update:   A22 -= Y L21^T on the lower 64 x 64 tiles (FP64).
+//   k_dense_update:   A22 -= Y L21^T on the lower 16 x 16 tiles (FP64).
 // A division by a pivot is a multiplication by its reciprocal.
 // Included by the translation units that launch them (internal linkage).
 #pragma once
@@ -256,28 +256,35 @@ __global__ void __launch_bounds__(ROWS) k_dense_panel_t(T* __restrict__ S0, T* _
 // column c's value reaches the other lanes by shuffle.  The dependency chain
 // of a row is 64 steps long instead of 2016 multiply-adds, which is what counts
 // for few rows (and in FP64, whose dependent multiply-add latency is long).
-template <class T>
-__global__ void __launch_bounds__(256) k_dense_panel_w(T* __restrict__ S0, T* __restrict__ Y0, int n, int k0,
+// From column 32 on only y_{l+32} is left to update.  WARPS rows per CTA.
+template <class T, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS) k_dense_panel_w(T* __restrict__ S0, T* __restrict__ Y0, int n, int k0,
                                                        int kb, int rend, int64_t bstride, int64_t ystride,
                                                        Tf32Images img) {
   __shared__ T L11[kPanelW][kPanelW + 1];
   __shared__ T dinv[kPanelW];
   T* S = S0 + (int64_t)blockIdx.y * bstride;
   T* Y = Y0 + (int64_t)blockIdx.y * ystride;
-  for (int q = threadIdx.x; q < kb * kb; q += blockDim.x) {
-    const int j = q / kb, i = q - j * kb;
-    L11[i][j] = S[(int64_t)(k0 + i) + (int64_t)(k0 + j) * n];
-  }
-  for (int c = threadIdx.x; c < kb; c += blockDim.x) dinv[c] = T(1) / S[(int64_t)(k0 + c) + (int64_t)(k0 + c) * n];
-  __syncthreads();
   const int lane = threadIdx.x & 31;
-  const int row = k0 + kb + blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-  if (row >= rend) return;
-  T y0 = lane < kb ? S[row + (int64_t)(k0 + lane) * n] : T(0);
-  T y1 = lane + 32 < kb ? S[row + (int64_t)(k0 + lane + 32) * n] : T(0);
-  for (int c = 0; c < kb; c++) {
-    const T yc = __shfl_sync(0xffffffffu, c < 32 ? y0 : y1, c & 31);
+  const int row = k0 + kb + blockIdx.x * WARPS + (threadIdx.x >> 5);
+  const bool live = row < rend;
+  T y0 = live && lane < kb ? S[row + (int64_t)(k0 + lane) * n] : T(0);
+  T y1 = live && lane + 32 < kb ? S[row + (int64_t)(k0 + lane + 32) * n] : T(0);
+  for (int q = threadIdx.x; q < kPanelW * kPanelW; q += blockDim.x) {
+    const int j = q / kPanelW, i = q - j * kPanelW;
+    if (i < kb && j < i) L11[i][j] = S[(int64_t)(k0 + i) + (int64_t)(k0 + j) * n];
+  }
+  for (int c = threadIdx.x; c < kb; c += blockDim.x) dinv[c] = pivot_recip(S[(int64_t)(k0 + c) + (int64_t)(k0 + c) * n]);
+  __syncthreads();
+  if (!live) return;
+  const int k32 = min(kb, 32);
+  for (int c = 0; c < k32; c++) {
+    const T yc = __shfl_sync(0xffffffffu, y0, c);
     if (lane > c && lane < kb) y0 -= yc * L11[lane][c];
+    if (lane + 32 < kb) y1 -= yc * L11[lane + 32][c];
+  }
+  for (int c = 32; c < kb; c++) {
+    const T yc = __shfl_sync(0xffffffffu, y1, c - 32);
     if (lane + 32 > c && lane + 32 < kb) y1 -= yc * L11[lane + 32][c];
   }
   if (lane < kb) {
@@ -327,82 +334,99 @@ inline void launch_dense_diag(T* S, int n, int k0, int kb, int nb, int64_t bstri
 }
 
 // Rows below the diagonal block of nb matrices.  A thread per row issues the
-// fewest instructions (no idle lanes) but its dependency chain is long; a
-// warp per row has a 64-step chain.  FP32 takes a thread per row from 2048
-// rows on.  In FP64 a warp issues one multiply-add per 64 cycles, so a thread
-// per row pays off once there are enough rows (m * nb >= 32768, over 1000
-// warps) to keep every sub-partition's FP64 pipe busy.
+// fewest instructions (no idle lanes) but its dependency chain is long (88 us
+// in FP64, 14 in FP32); a warp per row has a 64-step chain.  FP64: 200 rows
+// take 10.4 us with four warps per CTA, 12.4 with eight, 88 with a thread per
+// row; 14,400 rows 92, 88 and 88; 57,600 rows 337, 328 and 229.  FP32: 4,096
+// rows 12.3 us with a warp per row, 13.8 with a thread; 9,000 rows 16.5 and
+// 14.4.
+constexpr int kPanelRowsFour = 152 * 32;     // FP64: up to these rows, four warps per CTA
+constexpr int kPanelRowsThread = 152 * 96;   // FP64: from these rows on, a thread per row
+constexpr int kPanelRowsThreadF32 = 6144;    // FP32
 template <class T>
 inline void launch_dense_panel(T* S, T* Y, int n, int k0, int kb, int rend, int nb, int64_t bstride,
                                int64_t ystride, cudaStream_t st, int prio = 0, Tf32Images img = Tf32Images{}) {
   const int m = rend - k0 - kb;
   if (m <= 0) return;
   if constexpr (sizeof(T) == 4) {
-    if (m > 2048) {
+    if ((int64_t)m * nb >= kPanelRowsThreadF32) {
       launch_prio(k_dense_panel_t<T, 128>, dim3((m + 127) / 128, nb), dim3(128), 0, st, prio, S, Y, n, k0, kb,
                   rend, bstride, ystride, img);
       return;
     }
   } else {
-    if ((int64_t)m * nb >= 32768) {
+    if ((int64_t)m * nb >= kPanelRowsThread) {
       launch_prio(k_dense_panel_t<T, 32>, dim3((m + 31) / 32, nb), dim3(32), 0, st, prio, S, Y, n, k0, kb, rend,
                   bstride, ystride, img);
       return;
     }
   }
-  launch_prio(k_dense_panel_w<T>, dim3((m + 7) / 8, nb), dim3(256), 0, st, prio, S, Y, n, k0, kb, rend, bstride,
-              ystride, img);
+  if (sizeof(T) == 8 && (int64_t)m * nb <= kPanelRowsFour)
+    launch_prio(k_dense_panel_w<T, 4>, dim3((m + 3) / 4, nb), dim3(128), 0, st, prio, S, Y, n, k0, kb, rend, bstride,
+                ystride, img);
+  else
+    launch_prio(k_dense_panel_w<T, 8>, dim3((m + 7) / 8, nb), dim3(256), 0, st, prio, S, Y, n, k0, kb, rend, bstride,
+                ystride, img);
 }
 
-// Trailing update of matrix blockIdx.y on the lower 64 x 64 tiles below the
-// panel: A[i][j] -= sum_c Y[i][c] L[j][c] for k0+kb <= j <= i < rend.
-__global__ void __launch_bounds__(256) k_dense_update(double* __restrict__ S0, const double* __restrict__ Y0,
-                                                      int n, int k0, int kb, int rend, int64_t bstride,
-                                                      int64_t ystride) {
-  double* S = S0 + (int64_t)blockIdx.y * bstride;
-  const double* Y = Y0 + (int64_t)blockIdx.y * ystride;
+// Trailing update of matrix blockIdx.y on the lower 16 x 16 tiles below the
+// panel, one entry per thread: A[i][j] -= sum_c Y[i][c] L[j][c] for
+// k0+kb <= j <= i < rend.  What bounds it: the FP64 pipe, at two multiply-adds
+// per SM and cycle so narrow that two shared-memory loads per multiply-add hide
+// behind it; register tiles buy nothing, and 64 x 64 tiles cost a narrow
+// trailing matrix the chip (one such tile keeps its SM 63 us).  One matrix with
+// 200 rows: 8 us (64 x 64 tiles: 78); 96 matrices with 800 rows, 3.9 GFLOP:
+// 3.30 ms, 0.95 of the FP64 rate (3.78).
+constexpr int kUpdTile = 16;
+
+template <class T>
+__global__ void __launch_bounds__(kUpdTile * kUpdTile)
+    k_dense_update(T* __restrict__ S0, const T* __restrict__ Y0, int n, int k0, int kb, int rend,
+                         int64_t bstride, int64_t ystride) {
+  __shared__ T Ys[kPanelW][kUpdTile + 1];
+  __shared__ T Ls[kPanelW][kUpdTile + 1];
+  T* S = S0 + (int64_t)blockIdx.y * bstride;
+  const T* Y = Y0 + (int64_t)blockIdx.y * ystride;
   const int base = k0 + kb;
-  int tile = blockIdx.x, ti = 0;
-  while (tile > ti) {
-    tile -= ti + 1;
-    ti++;
+  // tile (ti, tj), tj <= ti, of the packed lower triangle
+  const int t = blockIdx.x;
+  int ti = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+  while (ti * (ti + 1) / 2 > t) ti--;
+  while ((ti + 1) * (ti + 2) / 2 <= t) ti++;
+  const int i0 = base + ti * kUpdTile, j0 = base + (t - ti * (ti + 1) / 2) * kUpdTile;
+  const int r = threadIdx.x % kUpdTile, g = threadIdx.x / kUpdTile;
+  T ys[kPanelW / kUpdTile], ls[kPanelW / kUpdTile];  // all loads first
+#pragma unroll
+  for (int u = 0; u < kPanelW / kUpdTile; u++) {
+    const int c = g + u * kUpdTile;
+    ys[u] = c < kb && i0 + r < rend ? Y[(i0 + r) + (int64_t)c * n] : T(0);
+    ls[u] = c < kb && j0 + r < rend ? S[(j0 + r) + (int64_t)(k0 + c) * n] : T(0);
   }
-  const int tj = tile;
-  const int i0 = base + ti * 64, j0 = base + tj * 64;
-  constexpr int KC = 32;              // columns staged per pass
-  __shared__ double Ys[KC][64 + 1];  // [c][i]
-  __shared__ double Ls[KC][64 + 1];  // [c][j]
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;  // 16 x 16, 4x4 outputs each
-  double acc[4][4] = {};
-  for (int cb = 0; cb < kb; cb += KC) {
-    const int kc = min(KC, kb - cb);
-    __syncthreads();
-    for (int q = threadIdx.x; q < kc * 64; q += 256) {
-      const int c = q / 64, r = q % 64;
-      Ys[c][r] = (i0 + r < rend) ? Y[(i0 + r) + (int64_t)(cb + c) * n] : 0.0;
-      Ls[c][r] = (j0 + r < rend) ? S[(j0 + r) + (int64_t)(k0 + cb + c) * n] : 0.0;
-    }
-    __syncthreads();
-    for (int c = 0; c < kc; c++) {
-      double a[4], bb[4];
+  const int i = i0 + r, j = j0 + g;  // consecutive threads, consecutive rows
+  const bool live = i < rend && j <= i;
+  const T cur = live ? S[i + (int64_t)j * n] : T(0);
 #pragma unroll
-      for (int u = 0; u < 4; u++) {
-        a[u] = Ys[c][ty + 16 * u];
-        bb[u] = Ls[c][tx + 16 * u];
-      }
-#pragma unroll
-      for (int u = 0; u < 4; u++)
-#pragma unroll
-        for (int v = 0; v < 4; v++) acc[u][v] += a[u] * bb[v];
-    }
+  for (int u = 0; u < kPanelW / kUpdTile; u++) {
+    Ys[g + u * kUpdTile][r] = ys[u];
+    Ls[g + u * kUpdTile][r] = ls[u];
   }
-#pragma unroll
-  for (int u = 0; u < 4; u++)
-#pragma unroll
-    for (int v = 0; v < 4; v++) {
-      const int i = i0 + ty + 16 * u, j = j0 + tx + 16 * v;
-      if (i < rend && j < rend && i >= j) S[i + (int64_t)j * n] -= acc[u][v];
-    }
+  __syncthreads();
+  T acc = T(0);
+  if (kb == kPanelW) {
+#pragma unroll 16
+    for (int c = 0; c < kPanelW; c++) acc += Ys[c][r] * Ls[c][g];
+  } else {
+    for (int c = 0; c < kb; c++) acc += Ys[c][r] * Ls[c][g];
+  }
+  if (live) S[i + (int64_t)j * n] = cur - acc;
+}
+
+template <class T>
+inline void launch_dense_update(T* S, const T* Y, int n, int k0, int kb, int rend, int nb, int64_t bstride,
+                                int64_t ystride, cudaStream_t st) {
+  const int tiles = (rend - k0 - kb + kUpdTile - 1) / kUpdTile;
+  k_dense_update<T><<<dim3(tiles * (tiles + 1) / 2, nb), kUpdTile * kUpdTile, 0, st>>>(S, Y, n, k0, kb, rend, bstride,
+                                                                                       ystride);
 }
 
 }  // namespace

@@ -243,9 +243,8 @@ cudaError_t launch_dense_tail(Handle& h, cudaStream_t st) {
     const int rest = nTa - k0 - kb;
     if (rest > 0) {
       launch_dense_panel<double>(h.Tt, h.TY, nTa, k0, kb, nTa, N, t2, ys, st);
-      const int tiles = (rest + 63) / 64;
       const int kt = kt_begin(h, kFamDenseF64, N * update_flops(rest, 0, rest, kb), st);
-      k_dense_update<<<dim3(tiles * (tiles + 1) / 2, N), 256, 0, st>>>(h.Tt, h.TY, nTa, k0, kb, nTa, t2, ys);
+      launch_dense_update<double>(h.Tt, h.TY, nTa, k0, kb, nTa, N, t2, ys, st);
       kt_end(h, kt, st);
       h.launches += 2;
     }

@@ -68,7 +68,7 @@ void free_all(Handle* h) {
                   h->t_scaleA, h->t_scaleB, h->Lx, h->LDx, h->a_vals, h->b_vals,
                   h->c_vals, h->anorm, h->W, h->G, h->S, h->Ypanel, h->knorm, h->counters, h->r,
                   h->z, h->u, h->v, h->tg, h->xg, h->x, h->dx, h->rho, h->rhs, h->red,
-                  h->trsv_flags, h->trsv_ticket, h->dev_err, h->S32, h->Y32, h->tw_img, h->ew_s_Y, h->ew_s_A,
+                  h->Zs, h->trsv_s, h->trsv_t, h->dev_err, h->S32, h->Y32, h->tw_img, h->ew_s_Y, h->ew_s_A,
                   h->ew_s_B, h->ew_s_scale, h->ew_t_Y, h->ew_t_A, h->ew_t_B, h->ew_t_scale, h->tc_imgA,
                   h->tc_imgB, h->tc_scaleA, h->tc_scaleB, h->gm_V, h->gm_Z, h->d.cum_y_ptr, h->d.cum_y_t,
                   h->d.cum_y_e, h->d.cum_z_ptr, h->d.cum_z_t, h->d.cum_z_e, h->d.cum_check, h->cum_err,
@@ -686,7 +686,10 @@ kkt_status analyze_one(const kkt_pattern* pat, const kkt_options* opt, double ta
     AL(gm_V, double, (int64_t)(m + 1) * nK);
     AL(gm_Z, double, (int64_t)m * nK);
   }
-  AL(trsv_flags, int, 2 * ((h->nC + kDenseNB - 1) / kDenseNB));
+  const int64_t nbS = (nCd + kDenseNB - 1) / kDenseNB, nbT = (h->nT + kDenseNB - 1) / kDenseNB;
+  AL(Zs, double, nbS > 1 ? 2 * nbS * kDenseNB * kDenseNB : 0);
+  AL(trsv_s, double, trsv_doubles(nbS, 2));
+  AL(trsv_t, double, trsv_doubles(nbT * h->N, 1));
   if ((h->opt.prec == KKT_TF32 || h->opt.prec == KKT_BF16) && !h->cum) {
     AL(S32, float, (int64_t)h->nC * h->nC);
     AL(Y32, float, (int64_t)h->nC * kDenseNB);
@@ -714,11 +717,8 @@ kkt_status analyze_one(const kkt_pattern* pat, const kkt_options* opt, double ta
       AL(ew_s_scale, double, 2 * ((int64_t)h->nC + 256));
     }
   }
-  AL(trsv_ticket, unsigned, 2);
   AL(dev_err, int, 1);
 #undef AL
-  if (e == cudaSuccess)
-    e = cudaMemset(h->trsv_flags, 0, sizeof(int) * (size_t)std::max(1, 2 * ((h->nC + kDenseNB - 1) / kDenseNB)));
   if (e == cudaSuccess) e = cudaMemset(h->dev_err, 0, sizeof(int));
   // W's structurally zero entries are never written: clear it once
   if (e == cudaSuccess) e = cudaMemset(h->W, 0, sizeof(double) * (size_t)std::max<int64_t>(1, (int64_t)C.nw * C.k * h->N));
@@ -869,7 +869,6 @@ void build_solve_graph(Handle& h) {
   cudaError_t e = cudaGraphCreate(&g, 0);
   if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&loop, g, 0, cudaGraphCondAssignDefault);
   const int64_t l0 = h.launches;
-  h.solve_capturing = true;
   auto capture_into = [&](cudaGraph_t target, bool prologue) -> cudaError_t {
     cudaError_t c = cudaStreamBeginCaptureToGraph(h.cap_stream, target, nullptr, nullptr, 0,
                                                   cudaStreamCaptureModeThreadLocal);
@@ -916,7 +915,6 @@ void build_solve_graph(Handle& h) {
     e = cudaGraphAddNode(&wnode, g, leaves.data(), nullptr, leaves.size(), &np);
     if (e == cudaSuccess) e = capture_into(np.conditional.phGraph_out[0], false);
   }
-  h.solve_capturing = false;
   h.launches = l0;
   if (e == cudaSuccess) e = cudaGraphInstantiate(&h.solve_exec[sf], g, 0);
   if (g) cudaGraphDestroy(g);

@@ -196,8 +196,9 @@ struct Handle {
   double* gm_V = nullptr;     // GMRES refinement: gmres_restart + 1 Krylov vectors of nK
   double* gm_Z = nullptr;     // and their preconditioned images (gmres_restart vectors)
   double* host_red = nullptr; // pinned
-  int* trsv_flags = nullptr;  // 2 * ceil(nC/64): block-ready epochs of the dense triangular solves
-  unsigned* trsv_ticket = nullptr;  // 2 tickets (forward, backward)
+  double* Zs = nullptr;       // 2 * ceil(nC/64) * 64 * 64: products that the solves with S fuse (dense.cu)
+  double* trsv_s = nullptr;   // publishing vectors and tickets of the dense triangular solves: of S
+  double* trsv_t = nullptr;   // and of the tails
   int* dev_err = nullptr;     // set when a bounded device wait runs out
   // device-side refinement (opt.device_refine): the solve graph and its loop state
   // (eta, eta_prev, steps, outcome: 0 converged, 1 stopped above the tolerance, 2 not finite)
@@ -205,7 +206,6 @@ struct Handle {
   // modes, or the FP64-accurate one, also after a fallback), built at first use
   cudaGraphExec_t solve_exec[2] = {nullptr, nullptr};
   bool solve_graph_failed[2] = {false, false};
-  bool solve_capturing = false;  // the dense triangular solves clear their flags instead of advancing an epoch
   double* rstate = nullptr;
   // structured S of the cumulative coupling (structured_s = 2, cumulative.cu):
   // ns x ns blocks, column-major, N of each unless noted
@@ -225,7 +225,6 @@ struct Handle {
   // FP32 copies of the period factors in the TF32/BF16 modes (the FP64 ones are the fallback)
   float *cum_Q32 = nullptr, *cum_QY32 = nullptr, *cum_Linv32 = nullptr, *cum_M32 = nullptr, *cum_Mt32 = nullptr;
   float* cum_D32 = nullptr;
-  int trsv_epoch = 1;          // the last epoch of a direct triangular solve of S (graph solves use 1)
   int64_t device_bytes = 0;
 
   bool factored = false;
@@ -310,6 +309,8 @@ cudaError_t launch_dense_solve(Handle& h, const double* t, double* x, cudaStream
 cudaError_t launch_dense_solve_f32(Handle& h, const double* t, double* x, cudaStream_t st);
 cudaError_t launch_diag_inverse(Handle& h, bool f32, cudaStream_t st);
 cudaError_t launch_tail_inverse(Handle& h, cudaStream_t st);
+cudaError_t launch_tail_trsv(Handle& h, bool forward, double* zt, cudaStream_t st);
+int64_t trsv_doubles(int64_t nb, int vectors);
 cudaError_t launch_tail_fsolve(Handle& h, double* z, cudaStream_t st);  // (tail.cu)
 cudaError_t launch_tail_bsolve(Handle& h, double* z, cudaStream_t st);
 // ---- (dense_tc.cu) ----

@@ -67,3 +67,64 @@ def test_factor_of_s_backward_error(n, prec):
     assert np.all(diff <= 4 * (n + 2) * u * (np.abs(lo) * np.abs(d) @ np.abs(lo).T))
     neg = int((np.linalg.eigvalsh(m) < 0).sum())
     assert info["n_neg"] == p.N * (p.nA - p.nP) + neg and info["n_zero"] == 0
+
+
+@pytest.mark.parametrize("prec,s", [("fp64", 0), ("fp64", 1), ("f64emu", 0), ("tf32", 0)])
+@pytest.mark.parametrize("n", [1, 63, 64, 65, 128, 129, 200, 577])
+def test_solve_with_s(n, prec, s):
+    """The chain of 64-row blocks of the triangular solves: with B = 0 the
+    coupling part of the solution is S^{-1} r_g alone.  The FP64-accurate
+    factors meet the backward error of the whole system (||K|| includes |S|)
+    without refinement: 4 (n + 2) u with the growth |L||D||L|^T <= 4 |S| of
+    these diagonally dominant matrices; the FP32 factor with it."""
+    torch = _torch()
+    import oracle
+    from paper_1907_05420_gb300 import binding as B
+
+    p, m = dense_c(n, 300 + n)
+    up = lambda v: torch.from_numpy(np.ascontiguousarray(v)).to("cuda:0")  # noqa: E731
+    r = up(p.rhs)
+    x = torch.full_like(r, float("nan"))
+    ref = prec != "tf32"
+    h = B.kkt_analyze(p, B.kkt_default_options(prec, structured_s=s, max_refine=0 if ref else 10, refine_tol=1e-13))
+    try:
+        B.kkt_factor(h, up(p.a_vals), up(p.b_vals), up(p.c_vals))
+        for _ in range(2):  # the second solve finds the first one's published vectors
+            B.kkt_solve(h, r, x)
+            eta = oracle.backward_error(p, x.cpu().numpy())
+            assert eta <= (16 * (n + 2) * 2.0 ** -53 if ref else 1e-13), eta
+    finally:
+        B.kkt_destroy(h)
+
+
+def test_solve_with_an_envelope_that_skips_blocks():
+    """A row block of S that starts left of a row block above it: the products
+    with the skipped blocks between them are zero."""
+    torch = _torch()
+    from dataclasses import replace
+
+    import oracle
+    from paper_1907_05420_gb300 import binding as B
+
+    p = make_problem(GridSpec(5, 6, 2, 1, 3, 1e-1, 1e1, 7, "tiny"))
+    n = 300
+    rng = np.random.default_rng(5)
+    cols = [[0, 200], [70, 290], [140, 150]]
+    b_row = np.full(6, p.nA - 1, dtype=np.int32)
+    p = replace(p, nC=n, c_vals=10.0 ** rng.uniform(-1, 1, n), b_blockptr=np.array([0, 2, 4, 6], np.int32), b_row=b_row,
+                b_col=np.array(sum(cols, []), np.int32), b_vals=rng.standard_normal(6),
+                rhs=rng.standard_normal(p.N * p.nA + n))
+    up = lambda v: torch.from_numpy(np.ascontiguousarray(v)).to("cuda:0")  # noqa: E731
+    xs = []
+    for s in (0, 1):
+        h = B.kkt_analyze(p, B.kkt_default_options("fp64", structured_s=s, max_refine=0, refine_tol=1e-14))
+        try:
+            r = up(p.rhs)
+            x = torch.full_like(r, float("nan"))
+            B.kkt_factor(h, up(p.a_vals), up(p.b_vals), up(p.c_vals))
+            B.kkt_solve(h, r, x)
+            xs.append(x.cpu().numpy())
+        finally:
+            B.kkt_destroy(h)
+        assert oracle.backward_error(p, xs[-1]) <= 1e-14
+    assert np.max(np.abs(xs[0] - xs[1])) <= 1e-10 * np.max(np.abs(xs[0]))

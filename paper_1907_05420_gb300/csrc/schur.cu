@@ -219,6 +219,41 @@ __global__ void k_assemble_s(const int64_t* __restrict__ s_key, const int64_t* _
   }
 }
 
+// The same with a warp per entry: lane l sums the records l, l + 32, ... and
+// the lanes add up in a fixed order.  An entry with many records (two coupling
+// columns that share rows in many blocks) is a chain of dependent gathers for a
+// thread, and its lanes read the records side by side.
+__global__ void __launch_bounds__(256) k_assemble_s_warp(
+    const int64_t* __restrict__ s_key, const int64_t* __restrict__ s_ptr, const int32_t* __restrict__ s_e1,
+    const int32_t* __restrict__ s_e2, const int32_t* __restrict__ e_t, const int32_t* __restrict__ e_block,
+    const double* __restrict__ b_vals, const double* __restrict__ G, int k, int64_t nkeys, int nC,
+    double* __restrict__ S) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; q < nkeys;
+       q += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    double acc = 0.0;
+    const int64_t r1 = s_ptr[q + 1];
+#pragma unroll 4
+    for (int64_t r = s_ptr[q] + lane; r < r1; r += 32) {
+      const int e1 = s_e1[r], e2 = s_e2[r];
+      const double* Gb = G + (int64_t)e_block[e1] * k * k;
+      acc += b_vals[e1] * b_vals[e2] * Gb[(int64_t)e_t[e1] * k + e_t[e2]];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) {
+      const int64_t key = s_key[q];
+      const int64_t c1 = key / nC, c2 = key - c1 * nC;
+      S[c1 + c2 * (int64_t)nC] -= acc;
+    }
+  }
+}
+
+// Records per entry of S from which a warp takes an entry.  SCOPF with 16
+// outages on 1,021 buses, 862 records per entry: 0.91 ms with a warp, 18.9 with a
+// thread; the adjacent coupling has one to four.
+constexpr int64_t kAssembleWarpRecords = 16;
+
 }  // namespace
 
 namespace {
@@ -303,12 +338,12 @@ cudaError_t launch_assemble_s(Handle& h, cudaStream_t st) {
   }
   const int64_t nkeys = (int64_t)h.cpl.s_key.size();
   if (nkeys > 0) {
-    int g2 = (int)std::min<int64_t>((nkeys + 255) / 256, 152 * 32);
-    {
-    k_assemble_s<<<g2, 256, 0, st>>>(h.d.s_key, h.d.s_ptr, h.d.s_e1, h.d.s_e2, h.d.e_t, h.d.e_block,
-                                     h.b_vals, h.G, h.cpl.k, nkeys, h.nC, h.S);
+    const bool warp = (int64_t)h.cpl.s_e1.size() >= kAssembleWarpRecords * nkeys;
+    const int g2 = (int)std::min<int64_t>((nkeys * (warp ? 32 : 1) + 255) / 256, 152 * 32);
+    (warp ? k_assemble_s_warp : k_assemble_s)<<<g2, 256, 0, st>>>(h.d.s_key, h.d.s_ptr, h.d.s_e1, h.d.s_e2, h.d.e_t,
+                                                                  h.d.e_block, h.b_vals, h.G, h.cpl.k, nkeys, h.nC,
+                                                                  h.S);
     h.launches++;
-  }
   }
   return cudaGetLastError();
 }

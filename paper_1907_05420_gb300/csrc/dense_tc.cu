@@ -158,28 +158,75 @@ __device__ __forceinline__ void emu_store_core_row(const double (&v)[8], int e_e
         make_uint4(packed[s][0], packed[s][1], packed[s][2], packed[s][3]);
 }
 
+// The largest of mag over the eight warps of a 256-thread CTA, per lane.
+__device__ __forceinline__ unsigned long long max_over_warps(unsigned long long mag, unsigned long long (&mx)[8][32]) {
+  mx[threadIdx.x >> 5][threadIdx.x & 31] = mag;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < 8; w++) mag = max(mag, mx[w][threadIdx.x & 31]);
+  return mag;
+}
+
+// Digit images of 32 rows of a 64-column operand by a CTA of 256 threads: lane
+// l takes row l, warp w the columns 8 w .. 8 w + 7 (one core row), read once
+// and side by side over the rows; the row's scale comes from the largest
+// magnitude of all eight warps.  src: the row's first column (leading dimension
+// n); columns >= kb and rows that are not live are zero; dst: the row's first
+// core row in the image, slices slice_stride apart.
+__device__ __forceinline__ void slice_rows64(const double* src, int64_t n, bool live, int kb, uint8_t* dst,
+                                             int slice_stride, double* scale, unsigned long long (&mx)[8][32],
+                                             const uint32_t* table) {
+  const int warp = threadIdx.x >> 5;
+  double v[8];
+  unsigned long long mag = 0;
+#pragma unroll
+  for (int e = 0; e < 8; e++) {
+    const int c = warp * 8 + e;
+    v[e] = live && c < kb ? src[(int64_t)c * n] : 0.0;
+    mag = max(mag, magnitude_bits(v[e]));
+  }
+  const int e_exp = scale_exponent(max_over_warps(mag, mx));
+  if (warp == 0) *scale = ldexp(1.0, e_exp);
+  emu_store_core_row(v, e_exp, table, dst + warp * 128, slice_stride);
+}
+
+// The operands of one 64-wide emulated update of matrix blockIdx.y: A = Y in
+// 128-row blocks (mpadA rows), then B = L21 in 64-row blocks, 32 rows per CTA
+// (see k_tc_slice for the rows).  One matrix of order 1,848: 3.7 us a step (15.5
+// with a thread per row that read its 64 columns twice), 24 of order 7,000: 44
+// us (61).
+__global__ void __launch_bounds__(256) k_emu_slice(const double* __restrict__ S0, const double* __restrict__ Y0, int n,
+                                                   int k0, int kb, int m, uint8_t* __restrict__ imgA0,
+                                                   uint8_t* __restrict__ imgB0, double* __restrict__ scaleA0,
+                                                   double* __restrict__ scaleB0, int mpadA, TcStrides ts) {
+  constexpr int KG = kgroups_of(2);
+  __shared__ unsigned long long mx[8][32];
+  __shared__ uint32_t bf16_of_byte[256];
+  bf16_of_byte[threadIdx.x] = bf16_bits_of_byte(threadIdx.x);
+  const int64_t bb = blockIdx.y;
+  const int q = blockIdx.x * 32 + (threadIdx.x & 31);
+  const bool isA = q < mpadA;
+  const int rho = isA ? q : q - mpadA, rows_blk = isA ? TM : TN, rr = rho % rows_blk;
+  const double* src = isA ? Y0 + bb * ts.y : S0 + bb * ts.s + (int64_t)k0 * n;  // Y columns 0.., L21 columns k0..
+  uint8_t* dst = (isA ? imgA0 + bb * ts.img_a : imgB0 + bb * ts.img_b) +
+                 (int64_t)(rho / rows_blk) * image_bytes(2, rows_blk) + (rr / 8) * KG * 128 + (rr % 8) * 16;
+  double* scale = (isA ? scaleA0 : scaleB0) + bb * ts.scale + rho;
+  __syncthreads();  // the table
+  slice_rows64(src + (k0 + kb + rho), n, rho < m, kb, dst, slice_bytes(2, rows_blk), scale, mx, bf16_of_byte);
+}
+
 template <int MODE, class T>
 __global__ void __launch_bounds__(256) k_tc_slice(const T* __restrict__ S0, const T* __restrict__ Y0,
                                                   int n, int k0, int kb, int m, uint8_t* __restrict__ imgA0,
-                                                  uint8_t* __restrict__ imgB0, double* __restrict__ scaleA0,
-                                                  double* __restrict__ scaleB0, int mpadA, int mpadB,
+                                                  uint8_t* __restrict__ imgB0, int mpadA, int mpadB,
                                                   TcStrides ts) {
+  static_assert(MODE != 2, "the emulated-FP64 operands are k_emu_slice's");
   const int64_t bb = blockIdx.y;
   const T* S = S0 + bb * ts.s;
   const T* Y = Y0 + bb * ts.y;
   uint8_t* imgA = imgA0 + bb * ts.img_a;
   uint8_t* imgB = imgB0 + bb * ts.img_b;
-  double* scaleA = scaleA0 + bb * ts.scale;
-  double* scaleB = scaleB0 + bb * ts.scale;
-  constexpr ModeCfg cfg = mode_cfg(MODE);
   constexpr int KG = kgroups_of(MODE);
-  constexpr int kpc = 16 / cfg.esz;  // elements per 16-byte core row
-  __shared__ uint32_t bf16_of_byte[256];
-  if (MODE == 2) {
-    for (int i = threadIdx.x; i < 256; i += blockDim.x)
-      bf16_of_byte[i] = bf16_bits_of_byte((uint32_t)i);
-    __syncthreads();
-  }
   const int base = k0 + kb;
   const int total = mpadA + mpadB;
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < total; q += gridDim.x * blockDim.x) {
@@ -192,52 +239,21 @@ __global__ void __launch_bounds__(256) k_tc_slice(const T* __restrict__ S0, cons
     const int blk = rho / rows_blk, rr = rho % rows_blk, g = rr / 8, r8 = rr % 8;
     uint8_t* blk_img = img + (int64_t)blk * image_bytes(MODE, rows_blk);
     const bool live = rho < m;
-    double e_scale = 1.0;
-    int e_exp = 0;
-    if (MODE == 2) {
-      // e = ilogb(max |v|) + 1 from the largest exponent field; rows whose
-      // largest entry is subnormal (or zero) take the FP64 route
-      int emax = 0;
-      if (live)
-        for (int c = 0; c < kb; c++) emax = max(emax, exp_field((double)src[(int64_t)(base + rho) + (col0 + c) * n]));
-      if (emax > 0) {
-        e_exp = emax - 1023 + 1;  // |v| < 2^e
-      } else {
-        double amax = 0.0;
-        if (live)
-          for (int c = 0; c < kb; c++) amax = fmax(amax, fabs((double)src[(int64_t)(base + rho) + (col0 + c) * n]));
-        e_exp = amax > 0.0 ? ilogb(amax) + 1 : 0;
-      }
-      e_scale = ldexp(1.0, e_exp);
-      if (isA) scaleA[rho] = e_scale;
-      else scaleB[rho] = e_scale;
-    }
     for (int kq = 0; kq < KG; kq++) {
-      // one 16-byte core row: elements kq*kpc .. kq*kpc+kpc-1
-      if (MODE == 2) {
-        // BF16 bit patterns of the signed digits, from the table of the 256
-        // byte values (no conversion instructions)
-        double v[8] = {};
-#pragma unroll
-        for (int e = 0; e < kpc; e++) {
-          const int c = kq * kpc + e;  // columns >= kb (a ragged panel) are zero
-          v[e] = (live && c < kb) ? (double)src[(int64_t)(base + rho) + (col0 + c) * n] : 0.0;
-        }
-        emu_store_core_row(v, e_exp, bf16_of_byte, blk_img + (g * KG + kq) * 128 + r8 * 16,
-                           slice_bytes(MODE, rows_blk));
-      } else if (MODE == 1) {
+      // one 16-byte core row: 8 BF16 or 4 TF32 elements (columns >= kb are zero)
+      if (MODE == 1) {
         __align__(16) __nv_bfloat16 h[8];
 #pragma unroll
         for (int e = 0; e < 8; e++)
-          h[e] = __float2bfloat16_rn((live && kq * kpc + e < kb)
-                                         ? (float)src[(int64_t)(base + rho) + (col0 + kq * kpc + e) * n]
+          h[e] = __float2bfloat16_rn((live && kq * 8 + e < kb)
+                                         ? (float)src[(int64_t)(base + rho) + (col0 + kq * 8 + e) * n]
                                          : 0.f);
         *reinterpret_cast<uint4*>(blk_img + (g * KG + kq) * 128 + r8 * 16) = *reinterpret_cast<const uint4*>(h);
       } else {
         __align__(16) float f[4];
 #pragma unroll
         for (int e = 0; e < 4; e++)
-          f[e] = (live && kq * kpc + e < kb) ? (float)src[(int64_t)(base + rho) + (col0 + kq * kpc + e) * n] : 0.f;
+          f[e] = (live && kq * 4 + e < kb) ? (float)src[(int64_t)(base + rho) + (col0 + kq * 4 + e) * n] : 0.f;
         *reinterpret_cast<uint4*>(blk_img + (g * KG + kq) * 128 + r8 * 16) = *reinterpret_cast<const uint4*>(f);
       }
     }
@@ -718,9 +734,8 @@ __global__ void __launch_bounds__(kEmuThreads, 1)
 // The panel of a step, Y = A21 L11^{-T} and L21 = Y D1^{-1} (the rows below
 // the diagonal block), as a product on the tensor cores instead of one
 // substitution per row on the FP64 pipe: W = L11^{-1} is formed per matrix
-// in FP64 (k_panel_inverse_slice, 64 x 64: column j of W by the substitution
-// that k_dense_panel_t runs for a row, applied to the unit vector e_j; the
-// same launch slices the rows of A21 into digits), and
+// in FP64 (k_panel_inverse_slice, 64 x 64; the same launch slices the rows of
+// A21 into digits), and
 // Y = A21 W^T is one 64-column product with K = 64 in the format of the
 // 64-wide emulated update (7 BF16 digit slices, 7 exact tensor-memory levels,
 // the same fold), written instead of accumulated (k_tc_panel_emu).  The
@@ -730,105 +745,134 @@ __global__ void __launch_bounds__(kEmuThreads, 1)
 // condition of the unit lower triangle L11, which the diagonal blocks of
 // these quasidefinite matrices keep small.
 
+// One doubling of the inversion in k_panel_inverse_slice: M holds, for every
+// pair of neighbouring h x h diagonal blocks of the unit lower triangle, their
+// inverses W11 and W22 (diagonals included) and L21 below W11; L21 becomes
+// W21 = -W22 (L21 W11).  256 threads, h / 8 entries each per product.
+template <int H>
+__device__ __forceinline__ void inverse_double(double (&M)[TK][TK + 1]) {
+  constexpr int PER = H / 8;
+  const int tid = threadIdx.x;
+  double t[PER];
+#pragma unroll
+  for (int u = 0; u < PER; u++) {  // T = L21 W11 (W11 lower: k >= j); neighbouring threads, neighbouring rows
+    const int e = tid + u * 256, b = e / (H * H) * 2 * H, j = e % (H * H) / H, i = e % H;
+    double acc = 0.0;
+    for (int k = j; k < H; k++) acc += M[b + H + i][b + k] * M[b + k][b + j];
+    t[u] = acc;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < PER; u++) {
+    const int e = tid + u * 256, b = e / (H * H) * 2 * H, j = e % (H * H) / H, i = e % H;
+    M[b + H + i][b + j] = t[u];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < PER; u++) {  // W21 = -W22 T (W22 lower: k <= i); neighbouring threads, neighbouring columns
+    const int e = tid + u * 256, b = e / (H * H) * 2 * H, i = e % (H * H) / H, j = e % H;
+    double acc = 0.0;
+    for (int k = 0; k <= i; k++) acc -= M[b + H + i][b + H + k] * M[b + H + k][b + j];
+    t[u] = acc;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < PER; u++) {
+    const int e = tid + u * 256, b = e / (H * H) * 2 * H, i = e % (H * H) / H, j = e % H;
+    M[b + H + i][b + j] = t[u];
+  }
+  __syncthreads();
+}
+
 // The two operands of k_tc_panel_emu for matrix blockIdx.y, in one launch.
 // CTA 0: W = L11^{-1} (the kb x kb unit lower triangle at (k0, k0) after
 // k_dense_diag_t) and the digit image of its rows, the B operand: row i of B
 // is row i of W (K index = column), rows and columns >= kb zero, the row
 // scales in scaleB[0..63].  CTAs 1..: the digit image of the rows of A21
 // (columns k0 .. k0 + kb of the rows below the diagonal block, rows >= m
-// zero), the A operand, with the row scales and layout of k_tc_slice.
+// zero), the A operand, 32 rows each, with the row scales and layout of
+// k_emu_slice.
+//
+// CTA 0 sets the launch's time for few matrices, on its SM's FP64 pipe: 64^3 / 6
+// multiply-adds, 11 us at best.  The 8 x 8 diagonal blocks are inverted by
+// substitution and then doubled three times with products that keep every
+// thread busy (inverse_double); a substitution of 64 columns by 64 threads is
+// one chain of 2016 multiply-adds.  One matrix of order 1,848: 22 us a launch
+// (90 with that substitution), 24 of order 7,000: 50 us (131).
 __global__ void __launch_bounds__(256) k_panel_inverse_slice(const double* __restrict__ S0, int n, int k0, int kb,
-                                                             int m, int mpadA, uint8_t* __restrict__ imgA0,
+                                                             int m, uint8_t* __restrict__ imgA0,
                                                              uint8_t* __restrict__ imgB0,
                                                              double* __restrict__ scaleA0,
                                                              double* __restrict__ scaleB0, TcStrides ts) {
   constexpr int KG = kgroups_of(2);
   __shared__ double M[TK][TK + 1];  // L11 by rows, then W by rows
+  __shared__ unsigned long long mx[8][32];
   __shared__ uint32_t bf16_of_byte[256];
   const int64_t bb = blockIdx.y;
   const double* S = S0 + bb * ts.s;
-  for (int i = threadIdx.x; i < 256; i += blockDim.x) bf16_of_byte[i] = bf16_bits_of_byte((uint32_t)i);
-  __syncthreads();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  bf16_of_byte[tid] = bf16_bits_of_byte(tid);
   if (blockIdx.x > 0) {
-    uint8_t* imgA = imgA0 + bb * ts.img_a;
-    double* scaleA = scaleA0 + bb * ts.scale;
-    for (int rho = (blockIdx.x - 1) * blockDim.x + threadIdx.x; rho < mpadA;
-         rho += (gridDim.x - 1) * blockDim.x) {
-      const bool live = rho < m;
-      const double* src = S + (int64_t)(k0 + kb + rho) + (int64_t)k0 * n;  // column c at src[c n]
-      // e = ilogb(max |v|) + 1 from the largest exponent field; rows whose
-      // largest entry is subnormal (or zero) take the FP64 route
-      int emax = 0;
-      if (live)
-        for (int c = 0; c < kb; c++) emax = max(emax, exp_field(src[(int64_t)c * n]));
-      int e_exp;
-      if (emax > 0) {
-        e_exp = emax - 1023 + 1;  // |v| < 2^e
-      } else {
-        double amax = 0.0;
-        if (live)
-          for (int c = 0; c < kb; c++) amax = fmax(amax, fabs(src[(int64_t)c * n]));
-        e_exp = amax > 0.0 ? ilogb(amax) + 1 : 0;
-      }
-      scaleA[rho] = ldexp(1.0, e_exp);
-      const int rr = rho % TM;
-      uint8_t* blk_img = imgA + (int64_t)(rho / TM) * image_bytes(2, TM) + (rr / 8) * KG * 128 + (rr % 8) * 16;
-      for (int kq = 0; kq < KG; kq++) {
-        double v[8];
-#pragma unroll
-        for (int e = 0; e < 8; e++) {
-          const int c = kq * 8 + e;
-          v[e] = (live && c < kb) ? src[(int64_t)c * n] : 0.0;
-        }
-        emu_store_core_row(v, e_exp, bf16_of_byte, blk_img + kq * 128, slice_bytes(2, TM));
-      }
-    }
+    const int rho = (blockIdx.x - 1) * 32 + lane, rr = rho % TM;
+    uint8_t* dst = imgA0 + bb * ts.img_a + (int64_t)(rho / TM) * image_bytes(2, TM) + (rr / 8) * KG * 128 +
+                   (rr % 8) * 16;
+    __syncthreads();  // the table
+    slice_rows64(S + (int64_t)(k0 + kb + rho) + (int64_t)k0 * n, n, rho < m, kb, dst, slice_bytes(2, TM),
+                 scaleA0 + bb * ts.scale + rho, mx, bf16_of_byte);
     return;
   }
-  uint8_t* imgB = imgB0 + bb * ts.img_b;
-  double* scaleB = scaleB0 + bb * ts.scale;
-  for (int q = threadIdx.x; q < TK * TK; q += blockDim.x) {
-    const int c = q / TK, j = q - c * TK;
-    M[j][c] = (j > c && j < kb) ? S[(int64_t)(k0 + j) + (int64_t)(k0 + c) * n] : 0.0;
+  {
+    double v[16];
+#pragma unroll
+    for (int u = 0; u < 16; u++) {
+      const int q = tid + u * 256, c = q / TK, j = q - c * TK;
+      v[u] = (j > c && j < kb) ? S[(int64_t)(k0 + j) + (int64_t)(k0 + c) * n] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < 16; u++) {
+      const int q = tid + u * 256, c = q / TK, j = q - c * TK;
+      M[j][c] = v[u];
+    }
   }
   __syncthreads();
-  // column jc of W: w L11^T = e_jc solved as a row, subtracted in increasing c
-  const int jc = threadIdx.x;
-  double w[TK];
+  // the 8 x 8 diagonal blocks: column jc of W, w L11^T = e_jc solved as a row
+  double w[8];
+  const int jc = tid, d8 = jc & ~7;
   if (jc < TK) {
 #pragma unroll
-    for (int c = 0; c < TK; c++) w[c] = (c == jc && c < kb) ? 1.0 : 0.0;
+    for (int c = 0; c < 8; c++) w[c] = (d8 + c == jc && jc < kb) ? 1.0 : 0.0;
 #pragma unroll
-    for (int j = 1; j < TK; j++) {
+    for (int j = 1; j < 8; j++) {
       double acc = w[j];
 #pragma unroll
-      for (int c = 0; c < j; c++) acc -= w[c] * M[j][c];
+      for (int c = 0; c < j; c++) acc -= w[c] * M[d8 + j][d8 + c];
       w[j] = acc;
     }
   }
-  __syncthreads();  // every read of L11 is done
+  __syncthreads();  // every read of L11's diagonal blocks is done
   if (jc < TK) {
 #pragma unroll
-    for (int i = 0; i < TK; i++) M[i][jc] = w[i];
+    for (int i = 0; i < 8; i++) M[d8 + i][jc] = w[i];
   }
   __syncthreads();
-  // the digit image: 64 rows x 8 core rows of K, two per thread
-  for (int q = threadIdx.x; q < TK * KG; q += blockDim.x) {
-    const int i = q / KG, kq = q - i * KG;
-    int emax = 0;
-    double amax = 0.0;
-    for (int c = 0; c < TK; c++) {
-      emax = max(emax, exp_field(M[i][c]));
-      amax = fmax(amax, fabs(M[i][c]));
-    }
-    // |w| < 2^e; rows whose largest entry is subnormal (or zero) take ilogb
-    const int e_exp = emax > 0 ? emax - 1023 + 1 : (amax > 0.0 ? ilogb(amax) + 1 : 0);
-    if (kq == 0) scaleB[i] = ldexp(1.0, e_exp);
+  inverse_double<8>(M);
+  inverse_double<16>(M);
+  inverse_double<32>(M);
+  // the digit image: rows 32 h + lane, columns 8 warp .. 8 warp + 7
+  uint8_t* imgB = imgB0 + bb * ts.img_b;
+  for (int h = 0; h < 2; h++) {
+    const int i = h * 32 + lane;
     double v[8];
+    unsigned long long mag = 0;
 #pragma unroll
-    for (int e = 0; e < 8; e++) v[e] = M[i][kq * 8 + e];
-    emu_store_core_row(v, e_exp, bf16_of_byte, imgB + ((i / 8) * KG + kq) * 128 + (i % 8) * 16,
-                       slice_bytes(2, TN));
+    for (int e = 0; e < 8; e++) {
+      v[e] = M[i][warp * 8 + e];
+      mag = max(mag, magnitude_bits(v[e]));
+    }
+    const int e_exp = scale_exponent(max_over_warps(mag, mx));
+    if (warp == 0) scaleB0[bb * ts.scale + i] = ldexp(1.0, e_exp);
+    emu_store_core_row(v, e_exp, bf16_of_byte, imgB + ((i / 8) * KG + warp) * 128 + (i % 8) * 16, slice_bytes(2, TN));
+    __syncthreads();  // mx is used again
   }
 }
 
@@ -985,66 +1029,63 @@ __host__ __device__ constexpr int ew_smem_bytes() { return kEwStages * (kEwStage
 // rows rho in [0, mpad) of the outer trailing matrix of matrix blockIdx.y:
 // operand A = rows of Y (columns 0..kw-1 of Yw, leading dimension n), operand
 // B = rows of L (columns K0..K0+kw-1 of S); rows >= m and columns >= kw are zero.
-__global__ void __launch_bounds__(128) k_slice_wide(const double* __restrict__ S0, const double* __restrict__ Yw0,
+// 32 rows of one operand per CTA: lane l takes row l, warp w the K chunk w (32
+// columns), read once, all loads in flight together, and kept in registers
+// while the row's scale is found.  One matrix of order 1,848: 8.4 us (106 with a
+// thread per row that read its 256 columns twice), 24 of order 7,000: 108 us
+// (281).
+__global__ void __launch_bounds__(256, 2) k_slice_wide(const double* __restrict__ S0, const double* __restrict__ Yw0,
                                                     int n, int K0, int kw, int base, int m, int mpad,
                                                     uint8_t* __restrict__ imgA0, uint8_t* __restrict__ imgB0,
                                                     double* __restrict__ scaleA0, double* __restrict__ scaleB0,
                                                     int64_t s_stride, int64_t y_stride, int64_t img_stride,
                                                     int64_t scale_stride) {
-  const int64_t bb = blockIdx.y;
+  static_assert(kEwChunks == 8, "a warp per K chunk");
+  __shared__ unsigned long long mx[8][32];
   __shared__ uint32_t bf16_of_byte[256];
-  for (int i = threadIdx.x; i < 256; i += blockDim.x) bf16_of_byte[i] = bf16_bits_of_byte((uint32_t)i);
-  __syncthreads();
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= 2 * mpad) return;
+  const int64_t bb = blockIdx.y;
+  bf16_of_byte[threadIdx.x] = bf16_bits_of_byte(threadIdx.x);
+  const int k = threadIdx.x >> 5;  // K chunk
+  const int q = blockIdx.x * 32 + (threadIdx.x & 31);
   const bool isA = q < mpad;
   const int rho = isA ? q : q - mpad;
   const bool live = rho < m;
-  const double* src = isA ? Yw0 + bb * y_stride : S0 + bb * s_stride + (int64_t)K0 * n;  // column 0 of the operand
-  const int64_t row = (int64_t)base + rho;
-  uint8_t* img = (isA ? imgA0 : imgB0) + bb * img_stride;
-  // e = ilogb(max |v|) + 2, so that |v| < 2^(e-1); rows whose largest entry is
-  // subnormal or zero take the FP64 route
-  int emax = 0;
-  if (live)
-    for (int c = 0; c < kw; c++) emax = max(emax, exp_field(src[row + (int64_t)c * n]));
-  int e_exp;
-  if (emax > 0) {
-    e_exp = emax - 1023 + 2;
-  } else {
-    double amax = 0.0;
-    if (live)
-      for (int c = 0; c < kw; c++) amax = fmax(amax, fabs(src[row + (int64_t)c * n]));
-    e_exp = amax > 0.0 ? ilogb(amax) + 2 : 0;
+  const double* src = (isA ? Yw0 + bb * y_stride : S0 + bb * s_stride + (int64_t)K0 * n) + (base + rho);
+  double v[kEwChunk];
+  unsigned long long mag = 0;
+#pragma unroll
+  for (int e = 0; e < kEwChunk; e++) {
+    const int c = k * kEwChunk + e;
+    v[e] = live && c < kw ? src[(int64_t)c * n] : 0.0;
   }
-  (isA ? scaleA0 : scaleB0)[bb * scale_stride + rho] = ldexp(1.0, e_exp);
+#pragma unroll
+  for (int e = 0; e < kEwChunk; e++) mag = max(mag, magnitude_bits(v[e]));
+  mag = max_over_warps(mag, mx);  // (its barrier covers the table too)
+  const int e_exp = mag ? scale_exponent(mag) + 1 : 0;  // |v| < 2^(e-1)
+  if (k == 0) (isA ? scaleA0 : scaleB0)[bb * scale_stride + rho] = ldexp(1.0, e_exp);
   const int blk = rho >> 6, rr = rho & 63, g = rr >> 3, r8 = rr & 7;
-  uint8_t* bimg = img + (int64_t)blk * kEwBlockBytes + (g * 4) * 128 + r8 * 16;
-  for (int k = 0; k < kEwChunks; k++) {
+  uint8_t* bimg = (isA ? imgA0 : imgB0) + bb * img_stride + (int64_t)blk * kEwBlockBytes + (g * 4) * 128 + r8 * 16;
 #pragma unroll
-    for (int kq = 0; kq < 4; kq++) {
-      uint32_t packed[kEmuSlices][4];
+  for (int kq = 0; kq < 4; kq++) {
+    uint32_t packed[kEmuSlices][4];
 #pragma unroll
-      for (int e = 0; e < 8; e++) {
-        const int c = k * kEwChunk + kq * 8 + e;
-        const double v = (live && c < kw) ? src[row + (int64_t)c * n] : 0.0;
-        long long vb;
-        const unsigned long long a = digits7(v, e_exp, vb);
-        int d[kEmuSlices];
-        balanced7(a, d);
-        const uint32_t neg = vb < 0 ? 0x8000u : 0u;
+    for (int e = 0; e < 8; e++) {
+      long long vb;
+      const unsigned long long a = digits7(v[kq * 8 + e], e_exp, vb);
+      int d[kEmuSlices];
+      balanced7(a, d);
+      const uint32_t neg = vb < 0 ? 0x8000u : 0u;
 #pragma unroll
-        for (int sl = 0; sl < kEmuSlices; sl++) {
-          const int t = d[sl];
-          const uint32_t hbits = t == 0 ? 0u : (bf16_of_byte[t < 0 ? -t : t] | ((t < 0 ? 0x8000u : 0u) ^ neg));
-          packed[sl][e >> 1] = (e & 1) ? (packed[sl][e >> 1] | (hbits << 16)) : hbits;
-        }
+      for (int sl = 0; sl < kEmuSlices; sl++) {
+        const int t = d[sl];
+        const uint32_t hbits = t == 0 ? 0u : (bf16_of_byte[t < 0 ? -t : t] | ((t < 0 ? 0x8000u : 0u) ^ neg));
+        packed[sl][e >> 1] = (e & 1) ? (packed[sl][e >> 1] | (hbits << 16)) : hbits;
       }
-#pragma unroll
-      for (int sl = 0; sl < kEmuSlices; sl++)
-        *reinterpret_cast<uint4*>(bimg + ((int64_t)(k * kEmuSlices + sl)) * kEwPiece + kq * 128) =
-            make_uint4(packed[sl][0], packed[sl][1], packed[sl][2], packed[sl][3]);
     }
+#pragma unroll
+    for (int sl = 0; sl < kEmuSlices; sl++)
+      *reinterpret_cast<uint4*>(bimg + ((int64_t)(k * kEmuSlices + sl)) * kEwPiece + kq * 128) =
+          make_uint4(packed[sl][0], packed[sl][1], packed[sl][2], packed[sl][3]);
   }
 }
 
@@ -1553,9 +1594,14 @@ cudaError_t factor_tc(Handle& h, T* S, T* Y, int n, int npiv, int nb, const TcSt
     const int TI = (m + TM - 1) / TM, TJ = (m + TN - 1) / TN;
     const int mpadA = TI * TM, mpadB = TJ * TN;
     if (!fuse) {
-      const int sgrid = std::max(1, std::min((mpadA + mpadB + 255) / 256, 152 * 8 / nb));
-      launch_prio(k_tc_slice<MODE, T>, dim3(sgrid, nb), dim3(256), 0, st, prio, S, Y, n, k0, kb, m, imgA, imgB,
-                  scaleA, scaleB, mpadA, mpadB, ts);
+      if constexpr (MODE == 2) {
+        launch_prio(k_emu_slice, dim3((mpadA + mpadB) / 32, nb), dim3(256), 0, st, prio, (const double*)S,
+                    (const double*)Y, n, k0, kb, m, imgA, imgB, scaleA, scaleB, mpadA, ts);
+      } else {
+        const int sgrid = std::max(1, std::min((mpadA + mpadB + 255) / 256, 152 * 8 / nb));
+        launch_prio(k_tc_slice<MODE, T>, dim3(sgrid, nb), dim3(256), 0, st, prio, S, Y, n, k0, kb, m, imgA, imgB,
+                    mpadA, mpadB, ts);
+      }
       h.launches++;
     }
     int tiles = 0;
@@ -1653,9 +1699,8 @@ cudaError_t factor_emu_wide(Handle& h, double* S, int n, int npiv, int nb, const
         // below the diagonal block, columns k0 .. k0 + kb of S), Y = A21 W^T
         const int TIp = (m + TM - 1) / TM;
         const int kp = kt_begin(h, kFamPanelEmu, nb * (double)m * kb * (kb - 1), st);
-        const int pgrid = std::max(1, std::min((TIp * TM + 255) / 256, 152 * 8 / nb));
-        launch_prio(k_panel_inverse_slice, dim3(1 + pgrid, nb), dim3(256), 0, st, prio, (const double*)S, n, k0, kb,
-                    m, TIp * TM, imgA, imgB, scaleA, scaleB, ti);
+        launch_prio(k_panel_inverse_slice, dim3(1 + TIp * (TM / 32), nb), dim3(256), 0, st, prio, (const double*)S, n,
+                    k0, kb, m, imgA, imgB, scaleA, scaleB, ti);
         e = launch_prio(k_tc_panel_emu, dim3(TIp, nb), dim3(256), panel_emu_smem_bytes(), st, prio, S, Yc, n, k0, kb,
                         m, (const uint8_t*)imgA, (const uint8_t*)imgB, (const double*)scaleA, (const double*)scaleB,
                         h.dev_err, ti);
@@ -1667,9 +1712,8 @@ cudaError_t factor_emu_wide(Handle& h, double* S, int n, int npiv, int nb, const
       const int TJl = (K0 + Wb - (k0 + kb) + TN - 1) / TN;
       if (TJl <= 0) continue;
       const int TI = (m + TM - 1) / TM, mpadA = TI * TM, mpadB = TJl * TN;
-      const int sgrid = std::max(1, std::min((mpadA + mpadB + 255) / 256, 152 * 8 / nb));
-      launch_prio(k_tc_slice<2, double>, dim3(sgrid, nb), dim3(256), 0, st, prio, (const double*)S,
-                  (const double*)Yc, n, k0, kb, m, imgA, imgB, scaleA, scaleB, mpadA, mpadB, ti);
+      launch_prio(k_emu_slice, dim3((mpadA + mpadB) / 32, nb), dim3(256), 0, st, prio, (const double*)S,
+                  (const double*)Yc, n, k0, kb, m, imgA, imgB, scaleA, scaleB, mpadA, ti);
       h.launches++;
       int tasks = 0;
       for (int I = 0; I < TI; I++) tasks += emu_row_tasks(I, TJl, 0);
@@ -1689,7 +1733,7 @@ cudaError_t factor_emu_wide(Handle& h, double* S, int n, int npiv, int nb, const
       if (e != cudaSuccess) break;
     }
     const int TI = (m + TM - 1) / TM, TJ = (m + TN - 1) / TN, mpad = TI * TM;
-    launch_prio(k_slice_wide, dim3((2 * mpad + 127) / 128, nb), dim3(128), 0, st, prio, (const double*)S,
+    launch_prio(k_slice_wide, dim3(2 * mpad / 32, nb), dim3(256), 0, st, prio, (const double*)S,
                 (const double*)ew.Yw, n, K0, Wb, base, m, mpad, ew.A, ew.B, ew.sA, ew.sB, ts.s, ew.y_stride,
                 ew.img_stride, ew.scale_stride);
     h.launches++;

@@ -119,6 +119,17 @@ KKT_HD void balanced7(unsigned long long q, int (&d)[kEmuSlices]) {
 // Biased exponent field of a double (0 for zero and subnormals).
 KKT_HD int exp_field(double v) { return (int)((bits_of(v) >> 52) & 0x7FF); }
 
+// Bits of |v|: as unsigned integers they order like the magnitudes, so a row's
+// largest one is found without the FP64 pipe.
+KKT_HD unsigned long long magnitude_bits(double v) { return (unsigned long long)bits_of(v) & 0x7FFFFFFFFFFFFFFFull; }
+
+// The exponent e with 2^(e-1) <= |v| < 2^e of the magnitude with these bits
+// (normal or subnormal; 0 for zero).
+KKT_HD int scale_exponent(unsigned long long mag) {
+  const int E = (int)(mag >> 52);
+  return E ? E - 1023 + 1 : (mag ? (63 - clz64(mag)) - 1074 + 1 : 0);
+}
+
 // BF16 bit pattern of an integer 0 <= v < 256 (exact: 8 significant bits).
 KKT_HD uint32_t bf16_bits_of_byte(uint32_t v) {
   if (v == 0) return 0u;

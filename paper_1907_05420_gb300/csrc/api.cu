@@ -63,7 +63,7 @@ void free_all(Handle* h) {
                   h->d.b_blockptr, h->d.e_t, h->d.e_block, h->d.wpos, h->d.sn_wrow, h->d.w_dpos,
                   h->d.w_col, h->d.reach_lvl_sn, h->d.s_key, h->d.s_ptr, h->d.s_e1, h->d.s_e2,
                   h->d.t_ptr, h->d.t_e, h->d.bt_ptr, h->d.E, h->d.g_rows, h->d.trsv_jlo, h->d.trsv_jhi,
-                  h->d.flvl_sn, h->d.twork, h->d.upd_ntail, h->d.reach_lvl_sn_nt, h->d.tail_sn_list, h->d.tail_wrow, h->d.wt_ptr, h->d.wt_idx,
+                  h->d.flvl_sn, h->d.twork, h->d.tpairs, h->d.upd_ntail, h->d.reach_lvl_sn_nt, h->d.tail_sn_list, h->d.hv_off, h->d.hv_sn, h->d.hv_col, h->d.hv_pos, h->d.tail_wrow, h->d.wt_ptr, h->d.wt_idx,
                   h->d.g_key, h->d.g_ptr, h->d.g_row, h->Xinv, h->Sdinv, h->wdinv, h->Xtail, h->Tt, h->TY, h->t_imgA, h->t_imgB,
                   h->t_scaleA, h->t_scaleB, h->Lx, h->LDx, h->a_vals, h->b_vals,
                   h->c_vals, h->anorm, h->W, h->G, h->S, h->Ypanel, h->knorm, h->counters, h->r,
@@ -388,11 +388,33 @@ kkt_status analyze_one(const kkt_pattern* pat, const kkt_options* opt, double ta
   g_gather(S, C, h->tail_aug ? S.tail_sn : S.nsuper, g_key, g_ptr, g_row);
   h->g_nkeys = (int64_t)g_key.size();
 
+  // the emulated tail takes the updates of its heavy descendants as one product
+  std::vector<int32_t> hv_sn_list, hv_sn, hv_col, hv_pos;
+  std::vector<int64_t> hv_off;
+  std::vector<char> heavy(S.nsuper, 0);
+  if (h->tail_mode == 2 && emu_wide_applies(h->nT)) hv_sn_list = heavy_descendants(S, kHeavyMaxCols);
+  for (size_t q = 0; q < hv_sn_list.size(); q++) {
+    const int s = hv_sn_list[q];
+    const int64_t m = S.sn_rowptr[s + 1] - S.sn_rowptr[s];
+    heavy[s] = 1;
+    for (int c = 0; c < S.sn_first[s + 1] - S.sn_first[s]; c++) {
+      hv_off.push_back(S.sn_valoff[s] + c * m);
+      hv_sn.push_back((int32_t)q);
+      hv_col.push_back(c);
+    }
+    hv_pos.resize((q + 1) * (size_t)h->nT, -1);
+    for (int64_t i = 0; i < m; i++) {
+      const int row = S.sn_rows[S.sn_rowptr[s] + i];
+      if (row >= S.tail_col) hv_pos[q * (size_t)h->nT + (row - S.tail_col)] = (int32_t)i;
+    }
+  }
+  h->hv_cols = (int32_t)hv_off.size();
+
   // factor work items: 32-row tiles of every supernode outside the dense tail,
-  // grouped by level, then those of the tail supernodes; per item the updates
-  // that meet the tile, as (update index within s's list, rows [ia, ib) of the
+  // grouped by level; per item the updates that meet the tile, as (update index within s's list, rows [ia, ib) of the
   // descendant that land in the tile), from the item's offset to the next item's
   std::vector<int32_t> fwork, twork, flvl_sn;
+  std::vector<TailPair> tpairs;
   std::vector<UpdPair> fpairs;
   // algorithmic flops of the updates of each work item: descendant d adds w_d
   // multiply-adds to every target entry (row i, column j) of the tile with
@@ -420,9 +442,7 @@ kkt_status analyze_one(const kkt_pattern* pat, const kkt_options* opt, double ta
         const int32_t ia = S.upd_r0[u] + (int32_t)(std::lower_bound(rel, rel + nrel, lo) - rel);
         const int32_t ib = S.upd_r0[u] + (int32_t)(std::lower_bound(rel, rel + nrel, hi) - rel);
         const int dd = S.upd_src[u];
-        // the tail's own updates among its supernodes run in the dense tail factor
-        const bool counted = !(s >= S.tail_sn && u - S.upd_ptr[s] >= S.upd_ntail[s]);
-        if (counted && ia < ib) {
+        if (ia < ib) {
           UpdPair pr;
           pr.rel = S.upd_reloff[u];
           pr.val = S.sn_valoff[dd];
@@ -454,16 +474,78 @@ kkt_status analyze_one(const kkt_pattern* pat, const kkt_options* opt, double ta
     h->fwork_lvl_ptr[l + 1] = (int32_t)(fwork.size() / 4);
     h->flvl_ptr[l + 1] = (int32_t)flvl_sn.size();
   }
-  // a closing item after each list gives its last item the end of its updates
-  const auto close_items = [&](std::vector<int32_t>& items) {
-    items.insert(items.end(), {0, 0, 0, (int32_t)fpairs.size()});
-  };
-  close_items(fwork);
-  item_flops = 0.0;
-  for (int s = S.tail_sn; s < S.nsuper; s++) add_items(s, twork);
-  h->tupd_flops = item_flops;
-  h->tail_items = (int32_t)(twork.size() / 4);
-  close_items(twork);
+  // a closing item gives the list's last item the end of its updates
+  fwork.insert(fwork.end(), {0, 0, 0, (int32_t)fpairs.size()});
+  // the dense tail's updates from outside it (but for its heavy descendants),
+  // by tile of the dense triangle, in the order of the descendants
+  {
+    const int tcols = tail_tile_cols(h->nT);
+    const int ntr = (h->nT + kTailTileRows - 1) / kTailTileRows, ntc = (h->nT + tcols - 1) / tcols;
+    struct Run {
+      int32_t tile, first, count;  // rows of d in one tile row (or column)
+    };
+    std::vector<Run> rr, cr;
+    const auto runs = [&](const int32_t* r, int m, int width, std::vector<Run>& out) {
+      out.clear();
+      for (int i = 0; i < m;) {
+        int e = i;
+        const int t = (r[i] - S.tail_col) / width;
+        while (e < m && (r[e] - S.tail_col) / width == t) e++;
+        out.push_back({t, i, e - i});
+        i = e;
+      }
+    };
+    std::vector<int32_t> count((size_t)ntr * ntc + 1, 0);
+    double flops = 0.0;
+    // two passes over the descendants: the number of pairs per tile, then the pairs
+    for (int pass = 0; pass < 2; pass++) {
+      for (int dd = 0; dd < S.tail_sn; dd++) {
+        if (heavy[dd]) continue;
+        const int64_t q0 = S.sn_rowptr[dd], q1 = S.sn_rowptr[dd + 1];
+        const int32_t* first = std::lower_bound(S.sn_rows.data() + q0, S.sn_rows.data() + q1, S.tail_col);
+        const int64_t t0 = first - S.sn_rows.data();
+        const int m = (int)(q1 - t0), wd = S.sn_first[dd + 1] - S.sn_first[dd];
+        if (m == 0) continue;
+        if (pass == 0) flops += (double)wd * m * (m + 1.0);
+        runs(first, m, kTailTileRows, rr);
+        runs(first, m, tcols, cr);
+        for (const Run& r : rr)
+          for (const Run& c : cr) {
+            if (c.tile * tcols > r.tile * kTailTileRows + kTailTileRows - 1) break;  // above the diagonal
+            int32_t& n = count[(size_t)r.tile * ntc + c.tile];
+            if (pass == 0) {
+              n++;
+              continue;
+            }
+            TailPair pr{};
+            const int64_t o = S.sn_valoff[dd] + (t0 - q0);
+            pr.li = o + r.first;
+            pr.lj = o + c.first;
+            pr.ri = t0 + r.first;
+            pr.rj = t0 + c.first;
+            pr.md = (int32_t)(q1 - q0);
+            pr.wd = (uint16_t)wd;
+            pr.ni = (uint16_t)r.count;
+            pr.nj = (uint16_t)c.count;
+            pr.inv = 65536u / (uint32_t)r.count + 1u;
+            tpairs[n++] = pr;
+          }
+      }
+      if (pass == 0) {  // counts to offsets; the tiles that have pairs become the items
+        int32_t total = 0;
+        for (int t = 0; t < ntr * ntc; t++) {
+          const int32_t n = count[t];
+          if (n > 0) twork.insert(twork.end(), {t / ntc, t % ntc, total});
+          count[t] = total;
+          total += n;
+        }
+        h->tail_items = (int32_t)(twork.size() / 3);
+        twork.insert(twork.end(), {0, 0, total});
+        tpairs.resize(total);
+      }
+    }
+    h->tupd_flops = flops;
+  }
   // per-column pivot position and primal flag
   std::vector<int64_t> col_dpos(n);
   std::vector<int32_t> col_primal(n);
@@ -557,6 +639,7 @@ kkt_status analyze_one(const kkt_pattern* pat, const kkt_options* opt, double ta
   UP(fpairs, fpairs);
   UP(flvl_sn, flvl_sn);
   UP(twork, twork);
+  UP(tpairs, tpairs);
   UP(upd_ntail, S.upd_ntail);
   UP(full_rowptr, full_rowptr);
   UP(full_col, full_col);
@@ -573,6 +656,12 @@ kkt_status analyze_one(const kkt_pattern* pat, const kkt_options* opt, double ta
   UP(reach_lvl_sn, C.reach_lvl_sn);
   UP(reach_lvl_sn_nt, reach_lvl_sn_nt);
   UP(tail_sn_list, tail_sn_list);
+  if (h->hv_cols > 0) {
+    UP(hv_off, hv_off);
+    UP(hv_sn, hv_sn);
+    UP(hv_col, hv_col);
+    UP(hv_pos, hv_pos);
+  }
   UP(tail_wrow, tail_wrow);
   UP(wt_ptr, C.wt_ptr);
   UP(wt_idx, C.wt_idx);

@@ -1026,6 +1026,35 @@ constexpr int kEwStageB = kEmuSlices * kEwPiece;      // 64 rows, 28,672 bytes
 constexpr int kEwStages = 2;
 __host__ __device__ constexpr int ew_smem_bytes() { return kEwStages * (kEwStageA + kEwStageB); }  // 168 KB
 
+// The digit images of a thread's 32 columns (K chunk k) of row rho of an operand.
+__device__ __forceinline__ void slice_chunk(const double (&v)[kEwChunk], int e_exp, uint8_t* img, int rho, int k,
+                                            const uint32_t* table) {
+  const int blk = rho >> 6, rr = rho & 63, g = rr >> 3, r8 = rr & 7;
+  uint8_t* bimg = img + (int64_t)blk * kEwBlockBytes + (g * 4) * 128 + r8 * 16;
+#pragma unroll
+  for (int kq = 0; kq < 4; kq++) {
+    uint32_t packed[kEmuSlices][4];
+#pragma unroll
+    for (int e = 0; e < 8; e++) {
+      long long vb;
+      const unsigned long long a = digits7(v[kq * 8 + e], e_exp, vb);
+      int d[kEmuSlices];
+      balanced7(a, d);
+      const uint32_t neg = vb < 0 ? 0x8000u : 0u;
+#pragma unroll
+      for (int sl = 0; sl < kEmuSlices; sl++) {
+        const int t = d[sl];
+        const uint32_t hbits = t == 0 ? 0u : (table[t < 0 ? -t : t] | ((t < 0 ? 0x8000u : 0u) ^ neg));
+        packed[sl][e >> 1] = (e & 1) ? (packed[sl][e >> 1] | (hbits << 16)) : hbits;
+      }
+    }
+#pragma unroll
+    for (int sl = 0; sl < kEmuSlices; sl++)
+      *reinterpret_cast<uint4*>(bimg + ((int64_t)(k * kEmuSlices + sl)) * kEwPiece + kq * 128) =
+          make_uint4(packed[sl][0], packed[sl][1], packed[sl][2], packed[sl][3]);
+  }
+}
+
 // rows rho in [0, mpad) of the outer trailing matrix of matrix blockIdx.y:
 // operand A = rows of Y (columns 0..kw-1 of Yw, leading dimension n), operand
 // B = rows of L (columns K0..K0+kw-1 of S); rows >= m and columns >= kw are zero.
@@ -1063,30 +1092,54 @@ __global__ void __launch_bounds__(256, 2) k_slice_wide(const double* __restrict_
   mag = max_over_warps(mag, mx);  // (its barrier covers the table too)
   const int e_exp = mag ? scale_exponent(mag) + 1 : 0;  // |v| < 2^(e-1)
   if (k == 0) (isA ? scaleA0 : scaleB0)[bb * scale_stride + rho] = ldexp(1.0, e_exp);
-  const int blk = rho >> 6, rr = rho & 63, g = rr >> 3, r8 = rr & 7;
-  uint8_t* bimg = (isA ? imgA0 : imgB0) + bb * img_stride + (int64_t)blk * kEwBlockBytes + (g * 4) * 128 + r8 * 16;
+  slice_chunk(v, e_exp, (isA ? imgA0 : imgB0) + bb * img_stride, rho, k, bf16_of_byte);
+}
+
+// The operands of the tail's heavy update (matrix blockIdx.y), straight from the
+// panels of the heavy descendants: B = L, A = L D over their columns, rows = the
+// tail's nT rows (zero where a descendant has none).  A column with pivot d is
+// balanced by an exact power of two, L 2^h and L D 2^-h with 2^(2h) about |d|:
+// the row scales then follow |L_ik| |d_k|^(1/2), whose squares the diagonal
+// entries of the matrix bound, instead of the spread of the pivots.  32 rows of
+// one operand per CTA, as k_slice_wide.
+__global__ void __launch_bounds__(256, 2) k_slice_heavy(const double* __restrict__ Lx, int64_t pt,
+                                                     const double* __restrict__ LDx, int64_t ldt,
+                                                     const int64_t* __restrict__ off, const int32_t* __restrict__ sn,
+                                                     const int32_t* __restrict__ col, const int32_t* __restrict__ pos,
+                                                     int ncol, int nT, int mpad, uint8_t* __restrict__ imgA0,
+                                                     uint8_t* __restrict__ imgB0, double* __restrict__ scaleA0,
+                                                     double* __restrict__ scaleB0, int64_t img_stride,
+                                                     int64_t scale_stride) {
+  __shared__ unsigned long long mx[8][32];
+  __shared__ uint32_t bf16_of_byte[256];
+  const int64_t bb = blockIdx.y;
+  bf16_of_byte[threadIdx.x] = bf16_bits_of_byte(threadIdx.x);
+  const int k = threadIdx.x >> 5;  // K chunk
+  const int q = blockIdx.x * 32 + (threadIdx.x & 31);
+  const bool isA = q < mpad;
+  const int rho = isA ? q : q - mpad;
+  const double* L = Lx + bb * pt;
+  const double* P = isA ? LDx + bb * ldt : L;
+  double v[kEwChunk];
+  unsigned long long mag = 0;
 #pragma unroll
-  for (int kq = 0; kq < 4; kq++) {
-    uint32_t packed[kEmuSlices][4];
-#pragma unroll
-    for (int e = 0; e < 8; e++) {
-      long long vb;
-      const unsigned long long a = digits7(v[kq * 8 + e], e_exp, vb);
-      int d[kEmuSlices];
-      balanced7(a, d);
-      const uint32_t neg = vb < 0 ? 0x8000u : 0u;
-#pragma unroll
-      for (int sl = 0; sl < kEmuSlices; sl++) {
-        const int t = d[sl];
-        const uint32_t hbits = t == 0 ? 0u : (bf16_of_byte[t < 0 ? -t : t] | ((t < 0 ? 0x8000u : 0u) ^ neg));
-        packed[sl][e >> 1] = (e & 1) ? (packed[sl][e >> 1] | (hbits << 16)) : hbits;
+  for (int e = 0; e < kEwChunk; e++) {
+    const int c = k * kEwChunk + e;
+    v[e] = 0.0;
+    if (c < ncol && rho < nT) {
+      const int i = pos[(int64_t)sn[c] * nT + rho];
+      if (i >= 0) {
+        const int h = (((__double2hiint(L[off[c] + col[c]]) >> 20) & 0x7ff) - 1023) >> 1;
+        v[e] = P[off[c] + i] * __hiloint2double((1023 + (isA ? -h : h)) << 20, 0);
       }
     }
-#pragma unroll
-    for (int sl = 0; sl < kEmuSlices; sl++)
-      *reinterpret_cast<uint4*>(bimg + ((int64_t)(k * kEmuSlices + sl)) * kEwPiece + kq * 128) =
-          make_uint4(packed[sl][0], packed[sl][1], packed[sl][2], packed[sl][3]);
   }
+#pragma unroll
+  for (int e = 0; e < kEwChunk; e++) mag = max(mag, magnitude_bits(v[e]));
+  mag = max_over_warps(mag, mx);  // (its barrier covers the table too)
+  const int e_exp = mag ? scale_exponent(mag) + 1 : 0;  // |v| < 2^(e-1)
+  if (k == 0) (isA ? scaleA0 : scaleB0)[bb * scale_stride + rho] = ldexp(1.0, e_exp);
+  slice_chunk(v, e_exp, (isA ? imgA0 : imgB0) + bb * img_stride, rho, k, bf16_of_byte);
 }
 
 // The K = 256 emulated update: one CTA per run of up to kEmuRun tiles (I, J)
@@ -1953,6 +2006,32 @@ cudaError_t launch_dense_ldlt_tc(Handle& h, int mode, unsigned long long* counte
     e = factor_tc<1, float>(h, h.S32, h.Y32, n, n, 1, one, PivotRule{}, rend, counters, h.tc_imgA, h.tc_imgB,
                             h.tc_scaleA, h.tc_scaleB, st);
   return e != cudaSuccess ? e : launch_diag_inverse(h, true, st);
+}
+
+// The update of the dense tails by their heavy descendants as one product per
+// tail: most multiply-adds of the updates from outside the tail come from a few
+// supernodes with thousands of rows in it (9,241 buses: 0.89 of them from 9
+// supernodes with 156 columns), which the supernodal kernel runs on the FP64
+// pipe.  24 tails of order 6,938, 225 columns: 0.96 ms of slicing and 8.6 ms of
+// products for 58 ms of supernodal updates.
+cudaError_t launch_tail_heavy_update(Handle& h, cudaStream_t st) {
+  if (h.hv_cols == 0) return cudaSuccess;
+  const int nT = h.nT, nTa = h.nTa, N = h.N;
+  const int TI = (nT + TM - 1) / TM, TJ = (nT + TN - 1) / TN, mpad = TI * TM;
+  const int64_t is = emu_wide_image_bytes(nTa), ss = 2 * ((int64_t)nTa + 2 * TM);
+  double *sA = h.ew_t_scale, *sB = h.ew_t_scale + (nTa + 2 * TM);
+  k_slice_heavy<<<dim3(2 * mpad / 32, N), 256, 0, st>>>(h.Lx, h.sym.panel_total, h.LDx, h.ld_total, h.d.hv_off,
+                                                        h.d.hv_sn, h.d.hv_col, h.d.hv_pos, h.hv_cols, nT, mpad,
+                                                        h.ew_t_A, h.ew_t_B, sA, sB, is, ss);
+  int tasks = 0;
+  for (int I = 0; I < TI; I++) tasks += emu_row_tasks(I, TJ, 0, 4);
+  const int kt = kt_begin(h, kFamEmuWide, N * update_flops(nT, 0, nT, h.hv_cols), st);
+  k_tc_update_emu_wide<<<dim3(tasks, N), kEmuThreads, ew_smem_bytes(), st>>>(
+      h.Tt, nTa, 0, nT, TI, TJ, 0, (h.hv_cols + kEwChunk - 1) / kEwChunk, h.ew_t_A, h.ew_t_B, sA, sB,
+      (int64_t)nTa * nTa, is, ss, h.dev_err);
+  kt_end(h, kt, st);
+  h.launches += 2;
+  return cudaGetLastError();
 }
 
 // The dense tails of the N block factors in emulated FP64: the batched

@@ -17,8 +17,8 @@
 //     pivot_eps*max|A_i| is replaced by the expected-sign value and counted).
 // The top of the tree (the dense tail, a suffix of the supernodes) is left out
 // of the level loop: once the rest is factored, its updates from outside the
-// tail are applied (k_factor_update over the tail's lists) and the tail is factored as one
-// dense triangle per block (tail.cu).
+// tail are applied and the tail is factored as one dense triangle per block
+// (tail.cu).
 // Every entry is written by one thread in a fixed order: the result does not
 // depend on scheduling.
 #include "handle.h"
@@ -81,9 +81,7 @@ __global__ void k_block_absmax(const double* __restrict__ a_vals, int64_t nnzA,
 // update order) and subtracted from the panel once.  For each update the rows
 // of d that land in the tile ([ia, ib), listed per tile at analysis with only
 // the updates that meet it) and the rows that land in s's columns ([r0, r1))
-// are staged in shared memory, the latter pre-multiplied by D_d.  For the tail
-// supernodes the lists hold only the updates from descendants outside the
-// dense tail; their updates among themselves are the dense tail factor's.
+// are staged in shared memory, the latter pre-multiplied by D_d.
 constexpr int kTileRows = kFactorTileRows;
 constexpr int kFactorThreads = 128;
 
@@ -243,19 +241,11 @@ cudaError_t launch_factor_levels(Handle& h, cudaStream_t st) {
     }
   }
   if (h.nT > 0) {
-    // updates of the tail from the rest of the tree (all factored by now), then
-    // the dense factor of the tail; an augmented tail first takes the W rows
-    // outside the tail and its own rows Z
+    // the dense tail, its updates from the rest of the tree (all factored by now)
+    // first; an augmented tail needs the W rows outside the tail and its own rows Z
     if (h.tail_aug) {
       cudaError_t e = launch_w_solve_before_tail(h, st);
       if (e != cudaSuccess) return e;
-    }
-    if (h.tail_items > 0) {
-      dim3 grid(h.tail_items, h.N);
-      const int kt = kt_begin(h, kFamFactorUpd, h.N * h.tupd_flops, st);
-      k_factor_update<<<grid, kFactorThreads, 0, st>>>(h.d.twork, h.d.fpairs, h.d, h.Lx, pt, h.LDx, h.ld_total);
-      kt_end(h, kt, st);
-      h.launches++;
     }
     cudaError_t e = launch_dense_tail(h, st);
     if (e != cudaSuccess) return e;

@@ -36,6 +36,24 @@ struct UpdPair {
 };
 static_assert(sizeof(UpdPair) == 48, "UpdPair layout");
 
+// One update of a tile of the dense tail (kTailTileRows x tail_tile_cols) by a
+// descendant d outside it: the entries of d's rows in the tile's rows times
+// those in its columns.
+struct alignas(16) TailPair {
+  int64_t li, lj;       // offsets of the first of them in a block's panels (L) and in LDx (L D)
+  int64_t ri, rj;       // and of their row numbers in sn_rows
+  int32_t md;           // rows of d's panel
+  uint16_t wd, ni, nj;  // its columns; rows in the tile's rows and columns
+  uint16_t pad;
+  uint32_t inv;         // 65536 / ni + 1: q / ni is q inv >> 16 for q < 2048
+};
+static_assert(sizeof(TailPair) == 48, "TailPair layout");
+constexpr int kTailTileRows = 4;
+// Columns of a tile: wide tiles meet a descendant less often, narrow ones spread
+// a small tail over more warps.  48 tails of order 130: 60 us with 64 columns, 92
+// with 128; 96 of order 724: 1.55 and 1.50 ms; 24 of order 6,938: 16.5 and 13.4 ms.
+inline int tail_tile_cols(int nT) { return nT >= 512 ? 128 : 64; }
+
 // Device copies of the symbolic structures.
 struct DevSym {
   int32_t* sn_first = nullptr;
@@ -84,9 +102,17 @@ struct DevSym {
   int32_t* trsv_jlo = nullptr;     // envelope of S (structured mode): first column block of each row block
   int32_t* trsv_jhi = nullptr;     // one past the last row block of each column block
   int32_t* flvl_sn = nullptr;      // supernodes outside the dense tail, by level (block factor)
-  int32_t* twork = nullptr;        // factor work items of the dense-tail supernodes
+  int32_t* twork = nullptr;        // tiles of the dense tail with updates from outside: 3 ints, tile row, tile column, first pair
+  TailPair* tpairs = nullptr;
   int32_t* upd_ntail = nullptr;    // per supernode: leading updates from outside the tail
   int32_t* reach_lvl_sn_nt = nullptr;  // reach supernodes outside the tail, by level
+  // heavy descendants of the tail (heavy_descendants), per column: its offset in
+  // a block's panels, its supernode among them and its column there; per heavy
+  // supernode and tail row: the row's position in the panel (-1: none)
+  int64_t* hv_off = nullptr;
+  int32_t* hv_sn = nullptr;
+  int32_t* hv_col = nullptr;
+  int32_t* hv_pos = nullptr;
   int32_t* tail_sn_list = nullptr;     // the tail supernodes in the reach of E
   int32_t* tail_wrow = nullptr;        // per tail column: its W row (-1 outside the reach)
   int32_t* wt_ptr = nullptr;           // per supernode: the columns of W on it (wt_idx)
@@ -133,7 +159,8 @@ struct Handle {
   std::vector<int32_t> reach_lvl_ptr_nt;  // reach supernodes outside the tail per level
   std::vector<int32_t> reach_lvl_chunks, reach_lvl_chunks_nt;  // W solve: 32-column chunks per level
   int64_t g_nkeys = 0;                 // nonzero entries of the sparse contraction
-  int32_t tail_items = 0;              // factor work items of the tail supernodes
+  int32_t hv_cols = 0;                 // columns of the tail's heavy descendants (0: none)
+  int32_t tail_items = 0;              // tiles of the dense tail in d.twork
   std::vector<double> fupd_flops;      // algorithmic flops of one block's supernodal updates, per level
   double tupd_flops = 0.0;             // and of the tail's updates from outside it
 
@@ -293,6 +320,8 @@ cudaError_t launch_factor_levels(Handle& h, cudaStream_t st);
 // ---- (tail.cu) ----
 cudaError_t launch_dense_tail(Handle& h, cudaStream_t st);
 cudaError_t launch_tail_factor_emulated(Handle& h, cudaStream_t st);  // (dense_tc.cu)
+cudaError_t launch_tail_heavy_update(Handle& h, cudaStream_t st);     // (dense_tc.cu)
+constexpr int kHeavyMaxCols = 256;  // K of the 256-wide emulated update
 // ---- (schur.cu) ----
 cudaError_t launch_w_solve(Handle& h, cudaStream_t st);
 cudaError_t launch_w_solve_before_tail(Handle& h, cudaStream_t st);

@@ -683,6 +683,39 @@ void choose_tail(Symbolic& S, int32_t N, int64_t max_bytes, int32_t min_cols, do
   }
 }
 
+std::vector<int32_t> heavy_descendants(const Symbolic& S, int32_t max_cols) {
+  // A column of a descendant with m rows in the tail takes m^2 / 2
+  // multiply-adds, in the dense product nT^2 / 2, which the tensor cores do 36
+  // times as fast (24 tails of order 6,938: 1.35e13 a second, slicing included;
+  // the supernodal updates of descendants with many rows: 3.9e11), so the line
+  // lies at m = nT / 6.  The slicing and one more read and write of the tails
+  // have to be earned too: 96 tails of order 724 with 84 such columns gain
+  // nothing (0.69 ms saved, 0.63 paid; here a gain of some 290 columns), the 24
+  // large ones with 225 columns (2,600) go from 58 ms to 9.6.
+  const int32_t nT = S.n - S.tail_col;
+  std::vector<std::pair<int32_t, int32_t>> cand;  // (-rows in the tail, supernode)
+  for (int32_t s = 0; s < S.tail_sn; s++) {
+    const int32_t* r0 = S.sn_rows.data() + S.sn_rowptr[s];
+    const int32_t* r1 = S.sn_rows.data() + S.sn_rowptr[s + 1];
+    const int32_t m = (int32_t)(r1 - std::lower_bound(r0, r1, S.tail_col));
+    if (6 * (int64_t)m >= nT && m > 0) cand.push_back({-m, s});
+  }
+  std::sort(cand.begin(), cand.end());
+  std::vector<int32_t> out;
+  int32_t cols = 0;
+  double gain = -640.0 * nT * (double)nT;
+  for (const auto& c : cand) {
+    const int32_t w = S.sn_first[c.second + 1] - S.sn_first[c.second];
+    if (cols + w > max_cols) continue;
+    cols += w;
+    gain += w * (36.0 * c.first * (double)c.first - nT * (double)nT);
+    out.push_back(c.second);
+  }
+  if (gain <= 0.0) out.clear();
+  std::sort(out.begin(), out.end());
+  return out;
+}
+
 int32_t tail_w_rows(const Symbolic& S, const Coupling& C, std::vector<int32_t>& wrow_of_tail_col) {
   const int32_t nT = S.n - S.tail_col;
   wrow_of_tail_col.assign(nT, -1);

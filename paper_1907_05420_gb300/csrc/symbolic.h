@@ -80,6 +80,13 @@ struct Symbolic {
 constexpr double kTailRatio = 1.5;
 void choose_tail(Symbolic& S, int32_t N, int64_t max_bytes, int32_t min_cols, double ratio = kTailRatio);
 
+// Descendants outside the dense tail whose updates of it the tail's tensor-core
+// update applies as one dense product: those with so many rows in the tail that
+// the zeros the product carries along cost less than the FP64 update they
+// replace.  At most max_cols columns in all (the ones with the most rows
+// first); returned in increasing order, empty if there is nothing to gain.
+std::vector<int32_t> heavy_descendants(const Symbolic& S, int32_t max_cols);
+
 // Coupling analysis: B_i (COO per block) against the block factor.
 // With E the sorted union of the rows that carry a nonzero of some B_i
 // (k = |E| rows), B_i = E M_i and

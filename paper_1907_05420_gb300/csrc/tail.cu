@@ -8,9 +8,8 @@
 // tail included, done by the blocked dense kernels that factor S
 // (dense_kernels.cuh), batched over the N blocks.
 //
-// Per factor: the tail panels (A's values plus the updates from outside the
-// tail, applied by the level loop) are gathered into the zeroed dense
-// triangles; each 64-wide panel step factors the diagonal blocks of all N
+// Per factor: the tail panels (A's values) are gathered into the zeroed dense
+// triangles, which then take the updates from outside the tail; each 64-wide panel step factors the diagonal blocks of all N
 // triangles (with the static-pivot rule and the inertia counts of the sparse
 // panels), forms L21 and Y = L21 D, and updates the trailing triangles, in
 // FP64 on the CUDA cores (tail mode 1) or in emulated FP64 on the tensor cores
@@ -73,6 +72,82 @@ __global__ void k_tail_aug_rows(double* __restrict__ W, int nw, int k, double* _
     double* a = Tb + (int64_t)(nT + t) + (int64_t)j * nTa;
     if (TO_DENSE) *a = Wb[(int64_t)r * k + t];
     else Wb[(int64_t)r * k + t] = *a * Tb[(int64_t)j + (int64_t)j * nTa];
+  }
+}
+
+// The updates of the dense tails from the descendants outside them (all but the
+// heavy ones), T[i][j] -= sum_d sum_k L_d[i][k] D_d[k] L_d[j][k], one warp per
+// (4-row tile with updates, block): the warp walks the descendants that meet
+// the tile, sums their products into its own tile in shared memory (lanes over
+// the entries a descendant adds, operands straight from global memory, each
+// warp on its own: no barrier between descendants) and subtracts it from the
+// dense triangle at the end.
+// What bounds it: latency, about two round trips to L2 per descendant and tile,
+// hidden by 40 warps per SM with small tiles; then the FP64 pipe, which the few
+// entries of a descendant in a tile fill by a third.  The CTA-wide staging of
+// k_factor_update, with two barriers per descendant, took 138 us for 48 tails of
+// order 130 (60 here), 2.8 ms for 96 of order 724 (1.5) and, without their heavy
+// descendants, 56 ms for 24 of order 6,938 (13.4); loading the next descendant
+// ahead into registers cost more warps than it hid latency (39 ms).
+constexpr int kTailUpdWarps = 4;
+inline int tail_upd_smem(int cols) { return kTailUpdWarps * cols * (kTailTileRows + 1) * (int)sizeof(double); }
+
+template <int COLS>
+__global__ void __launch_bounds__(32 * kTailUpdWarps, 10)
+    k_tail_update(const int32_t* __restrict__ work, int nitems, const TailPair* __restrict__ pairs,
+                  const int32_t* __restrict__ sn_rows, const double* __restrict__ Lx, int64_t pt,
+                  const double* __restrict__ LDx, int64_t ldt, double* __restrict__ T, int nT, int nTa, int tail_col) {
+  extern __shared__ __align__(16) double accs[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, b = blockIdx.y;
+  const int item = blockIdx.x * kTailUpdWarps + warp;
+  if (item >= nitems) return;
+  double* acc = accs + warp * COLS * (kTailTileRows + 1);  // [column][row]
+  const int i0 = work[3 * item] * kTailTileRows, j0 = work[3 * item + 1] * COLS;
+  const int p0 = work[3 * item + 2], p1 = work[3 * item + 5];
+  for (int q = lane; q < COLS * (kTailTileRows + 1); q += 32) acc[q] = 0.0;
+  const double* Lb = Lx + b * pt;
+  const double* LDb = LDx + b * ldt;
+  const int ri0 = tail_col + i0, rj0 = tail_col + j0;
+  TailPair Rn = pairs[p0];
+  __syncwarp();
+  for (int p = p0; p < p1; p++) {
+    const TailPair R = Rn;
+    if (p + 1 < p1) Rn = pairs[p + 1];
+    const int ne = R.ni * R.nj, md = R.md, wd = R.wd;
+    for (int q = lane; q < ne; q += 32) {
+      const int j = (int)(((uint32_t)q * R.inv) >> 16), i = q - j * R.ni;
+      const int row = sn_rows[R.ri + i] - ri0, col = sn_rows[R.rj + j] - rj0;
+      const double* a = Lb + R.li + i;
+      const double* c = LDb + R.lj + j;
+      double sum = 0.0;
+      int k = 0;
+      for (; k + 4 <= wd; k += 4, a += 4 * md, c += 4 * md) {
+        const double a0 = a[0], a1 = a[md], a2 = a[2 * md], a3 = a[3 * md];
+        const double c0 = c[0], c1 = c[md], c2 = c[2 * md], c3 = c[3 * md];
+        sum += a0 * c0;
+        sum += a1 * c1;
+        sum += a2 * c2;
+        sum += a3 * c3;
+      }
+      if (k < wd) {  // one to three columns left, loaded together
+        const bool b1 = k + 1 < wd, b2 = k + 2 < wd;
+        const double a0 = a[0], a1 = b1 ? a[md] : 0.0, a2 = b2 ? a[2 * md] : 0.0;
+        const double c0 = c[0], c1 = b1 ? c[md] : 0.0, c2 = b2 ? c[2 * md] : 0.0;
+        sum += a0 * c0;
+        if (b1) sum += a1 * c1;
+        if (b2) sum += a2 * c2;
+      }
+      if (i0 + row >= j0 + col) acc[col * (kTailTileRows + 1) + row] += sum;
+    }
+    __syncwarp();
+  }
+  double* Tb = T + (int64_t)b * nTa * nTa;
+  const int row = lane & (kTailTileRows - 1), i = i0 + row;
+  constexpr int kStep = 32 / kTailTileRows;
+#pragma unroll 8
+  for (int c = lane / kTailTileRows; c < COLS; c += kStep) {
+    const int j = j0 + c;
+    if (i < nT && j <= i) Tb[(int64_t)i + (int64_t)j * nTa] -= acc[c * (kTailTileRows + 1) + row];
   }
 }
 
@@ -146,8 +221,18 @@ cudaError_t launch_dense_tail(Handle& h, cudaStream_t st) {
     k_tail_aug_rows<true><<<agrid, 256, 0, st>>>(h.W, nw, k, h.Tt, nT, nTa, h.d.tail_wrow);
     h.launches++;
   }
+  if (h.tail_items > 0) {
+    const int kt = kt_begin(h, kFamFactorUpd, N * h.tupd_flops, st);
+    const int cols = tail_tile_cols(nT);
+    (cols == 128 ? k_tail_update<128> : k_tail_update<64>)<<<
+        dim3((h.tail_items + kTailUpdWarps - 1) / kTailUpdWarps, N), 32 * kTailUpdWarps, tail_upd_smem(cols), st>>>(
+        h.d.twork, h.tail_items, h.d.tpairs, h.d.sn_rows, h.Lx, pt, h.LDx, h.ld_total, h.Tt, nT, nTa, tail_col);
+    kt_end(h, kt, st);
+    h.launches++;
+  }
   if (h.tail_mode == 2) {
-    e = launch_tail_factor_emulated(h, st);
+    e = launch_tail_heavy_update(h, st);
+    if (e == cudaSuccess) e = launch_tail_factor_emulated(h, st);
     if (e != cudaSuccess) return e;
   }
   const PivotRule rule{h.anorm, h.opt.pivot_eps, h.d.col_primal + tail_col};

@@ -63,7 +63,7 @@ void free_all(Handle* h) {
                   h->d.b_blockptr, h->d.e_t, h->d.e_block, h->d.wpos, h->d.sn_wrow, h->d.w_dpos,
                   h->d.w_col, h->d.reach_lvl_sn, h->d.s_key, h->d.s_ptr, h->d.s_e1, h->d.s_e2,
                   h->d.t_ptr, h->d.t_e, h->d.bt_ptr, h->d.E, h->d.g_rows, h->d.trsv_jlo, h->d.trsv_jhi,
-                  h->d.flvl_sn, h->d.twork, h->d.tpairs, h->d.upd_ntail, h->d.reach_lvl_sn_nt, h->d.tail_sn_list, h->d.hv_off, h->d.hv_sn, h->d.hv_col, h->d.hv_pos, h->d.tail_wrow, h->d.wt_ptr, h->d.wt_idx,
+                  h->d.flvl_sn, h->d.flvl_desc, h->d.fr_ptr, h->d.fr_rec, h->d.wr_ptr, h->d.wr_row, h->d.w_sn, h->d.twork, h->d.tpairs, h->d.upd_ntail, h->d.reach_lvl_sn_nt, h->d.tail_sn_list, h->d.hv_off, h->d.hv_sn, h->d.hv_col, h->d.hv_pos, h->d.tail_wrow, h->d.wt_ptr, h->d.wt_idx,
                   h->d.g_key, h->d.g_ptr, h->d.g_row, h->Xinv, h->Sdinv, h->wdinv, h->Xtail, h->Tt, h->TY, h->t_imgA, h->t_imgB,
                   h->t_scaleA, h->t_scaleB, h->Lx, h->LDx, h->a_vals, h->b_vals,
                   h->c_vals, h->anorm, h->W, h->G, h->S, h->Ypanel, h->knorm, h->counters, h->r,
@@ -462,6 +462,10 @@ kkt_status analyze_one(const kkt_pattern* pat, const kkt_options* opt, double ta
   h->fwork_lvl_ptr.assign(S.nlevels + 1, 0);
   h->flvl_ptr.assign(S.nlevels + 1, 0);
   h->fupd_flops.assign(S.nlevels, 0.0);
+  h->flvl_small.assign(S.nlevels, 0);
+  const auto small_sn = [&](int s) {
+    return S.sn_first[s + 1] - S.sn_first[s] <= kSmallSnCols && S.sn_rowptr[s + 1] - S.sn_rowptr[s] <= kSmallSnRows;
+  };
   for (int l = 0; l < S.nlevels; l++) {
     item_flops = 0.0;
     for (int q = S.lvl_ptr[l]; q < S.lvl_ptr[l + 1]; q++) {
@@ -470,6 +474,8 @@ kkt_status analyze_one(const kkt_pattern* pat, const kkt_options* opt, double ta
       flvl_sn.push_back(s);
       add_items(s, fwork);
     }
+    const auto mid = std::stable_partition(flvl_sn.begin() + h->flvl_ptr[l], flvl_sn.end(), small_sn);
+    h->flvl_small[l] = (int32_t)(mid - flvl_sn.begin()) - h->flvl_ptr[l];
     h->fupd_flops[l] = item_flops;
     h->fwork_lvl_ptr[l + 1] = (int32_t)(fwork.size() / 4);
     h->flvl_ptr[l + 1] = (int32_t)flvl_sn.size();
@@ -545,6 +551,50 @@ kkt_status analyze_one(const kkt_pattern* pat, const kkt_options* opt, double ta
       }
     }
     h->tupd_flops = flops;
+  }
+  // the forward solve's lists: per row (in elimination order) its entries in
+  // the panels of the descendants outside the tail, in their order
+  std::vector<int64_t> fr_ptr(n + 1, 0);
+  std::vector<RowRec> fr_rec;
+  for (int pass = 0; pass < 2; pass++) {
+    std::vector<int64_t> at(fr_ptr.begin(), fr_ptr.end() - 1);
+    for (int s = 0; s < S.nsuper; s++)
+      for (int64_t u = S.upd_ptr[s]; u < S.upd_ptr[s + 1]; u++) {
+        const int dd = S.upd_src[u];
+        if (dd >= S.tail_sn) continue;
+        const int md = (int)(S.sn_rowptr[dd + 1] - S.sn_rowptr[dd]), fd = S.sn_first[dd];
+        for (int i = S.upd_r0[u]; i < S.upd_r1[u]; i++) {
+          const int j = S.sn_rows[S.sn_rowptr[dd] + i];
+          if (pass == 0) fr_ptr[j + 1]++;
+          else fr_rec[at[j]++] = RowRec{(S.sn_valoff[dd] + i) * 64 + (S.sn_first[dd + 1] - fd), md, fd};
+        }
+      }
+    if (pass == 0) {
+      for (int j = 0; j < n; j++) fr_ptr[j + 1] += fr_ptr[j];
+      fr_rec.resize(fr_ptr[n]);
+    }
+  }
+  std::vector<SnDesc> flvl_desc;
+  for (int s : flvl_sn)
+    flvl_desc.push_back(SnDesc{S.sn_valoff[s], S.sn_rowptr[s], S.sn_first[s], S.sn_first[s + 1] - S.sn_first[s],
+                               (int32_t)(S.sn_rowptr[s + 1] - S.sn_rowptr[s]), 0});
+  // W by structure outside the (augmented) tail: per column its nonzero rows
+  std::vector<int32_t> wr_ptr(C.k + 1, 0), wr_row, w_sn(C.nw, 0);
+  for (int s = 0; s < S.nsuper; s++) {
+    if (C.sn_wrow[s] < 0) continue;
+    const int w = S.sn_first[s + 1] - S.sn_first[s];
+    for (int c = 0; c < w; c++) w_sn[C.sn_wrow[s] + c] = s;
+    if (C.sn_wrow[s] < h->nw_nt)
+      for (int q = C.wt_ptr[s]; q < C.wt_ptr[s + 1]; q++) wr_ptr[C.wt_idx[q] + 1] += w;
+  }
+  for (int t = 0; t < C.k; t++) wr_ptr[t + 1] += wr_ptr[t];
+  wr_row.resize(wr_ptr[C.k]);
+  {
+    std::vector<int32_t> at(wr_ptr.begin(), wr_ptr.end() - 1);
+    for (int s = 0; s < S.nsuper; s++)
+      if (C.sn_wrow[s] >= 0 && C.sn_wrow[s] < h->nw_nt)
+        for (int q = C.wt_ptr[s]; q < C.wt_ptr[s + 1]; q++)
+          for (int c = 0; c < S.sn_first[s + 1] - S.sn_first[s]; c++) wr_row[at[C.wt_idx[q]]++] = C.sn_wrow[s] + c;
   }
   // per-column pivot position and primal flag
   std::vector<int64_t> col_dpos(n);
@@ -638,6 +688,12 @@ kkt_status analyze_one(const kkt_pattern* pat, const kkt_options* opt, double ta
   UP(fwork, fwork);
   UP(fpairs, fpairs);
   UP(flvl_sn, flvl_sn);
+  UP(flvl_desc, flvl_desc);
+  UP(fr_ptr, fr_ptr);
+  UP(fr_rec, fr_rec);
+  UP(wr_ptr, wr_ptr);
+  UP(wr_row, wr_row);
+  UP(w_sn, w_sn);
   UP(twork, twork);
   UP(tpairs, tpairs);
   UP(upd_ntail, S.upd_ntail);

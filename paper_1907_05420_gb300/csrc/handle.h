@@ -54,6 +54,23 @@ constexpr int kTailTileRows = 4;
 // with 128; 96 of order 724: 1.55 and 1.50 ms; 24 of order 6,938: 16.5 and 13.4 ms.
 inline int tail_tile_cols(int nT) { return nT >= 512 ? 128 : 64; }
 
+// One entry of a row's list for the forward solve: the row's entries in the panel
+// of a descendant outside the dense tail, columns fd .. fd + wd - 1.
+struct alignas(16) RowRec {
+  int64_t off_wd;  // offset in a block's panels (first column) * 64 + wd
+  int32_t md, fd;  // rows of the panel; its first column
+};
+static_assert(sizeof(RowRec) == 16 && kMaxSnWidth < 64, "RowRec layout");
+// A supernode outside the dense tail, in level order, for the solves.
+struct alignas(16) SnDesc {
+  int64_t val, rows;  // offsets of its panel and of its row list
+  int32_t f, w, m;    // first column, columns, rows
+  int32_t pad;
+};
+static_assert(sizeof(SnDesc) == 32, "SnDesc layout");
+// Supernodes that eight lanes solve with (at most this many columns and rows).
+constexpr int kSmallSnCols = 8, kSmallSnRows = 48;
+
 // Device copies of the symbolic structures.
 struct DevSym {
   int32_t* sn_first = nullptr;
@@ -101,6 +118,12 @@ struct DevSym {
   int32_t* g_rows = nullptr;       // W rows in contraction order: primal chunks, then multiplier chunks
   int32_t* trsv_jlo = nullptr;     // envelope of S (structured mode): first column block of each row block
   int32_t* trsv_jhi = nullptr;     // one past the last row block of each column block
+  SnDesc* flvl_desc = nullptr;     // the supernodes of flvl_sn
+  int64_t* fr_ptr = nullptr;       // per column: its row's records for the forward solve
+  RowRec* fr_rec = nullptr;
+  int32_t* wr_ptr = nullptr;       // per column of W: its nonzero rows outside the (augmented) tail
+  int32_t* wr_row = nullptr;
+  int32_t* w_sn = nullptr;         // per W row: its supernode
   int32_t* flvl_sn = nullptr;      // supernodes outside the dense tail, by level (block factor)
   int32_t* twork = nullptr;        // tiles of the dense tail with updates from outside: 3 ints, tile row, tile column, first pair
   TailPair* tpairs = nullptr;
@@ -149,6 +172,7 @@ struct Handle {
   std::vector<int32_t> reach_lvl_ptr;
   std::vector<int32_t> panel_rend;     // structured mode: per 64-wide panel, one past its last nonzero row
   std::vector<int32_t> flvl_ptr;       // supernodes outside the dense tail per level (factor)
+  std::vector<int32_t> flvl_small;     // and how many of them, the first ones, are small (kSmallSnCols, kSmallSnRows)
   int32_t nT = 0;                      // columns of the dense tail (0 = none)
   double tail_ratio = 0.0;             // cost ratio the tail was chosen with
   double last_delta_w = 0.0;           // inertia correction: the last successful shift > 0 (0: none yet)
@@ -340,7 +364,7 @@ cudaError_t launch_diag_inverse(Handle& h, bool f32, cudaStream_t st);
 cudaError_t launch_tail_inverse(Handle& h, cudaStream_t st);
 cudaError_t launch_tail_trsv(Handle& h, bool forward, double* zt, cudaStream_t st);
 int64_t trsv_doubles(int64_t nb, int vectors);
-cudaError_t launch_tail_fsolve(Handle& h, double* z, cudaStream_t st);  // (tail.cu)
+cudaError_t launch_tail_fsolve(Handle& h, double* z, cudaStream_t st);  // (solve.cu)
 cudaError_t launch_tail_bsolve(Handle& h, double* z, cudaStream_t st);
 // ---- (dense_tc.cu) ----
 cudaError_t launch_dense_ldlt_tc(Handle& h, int mode, unsigned long long* counters, cudaStream_t st);

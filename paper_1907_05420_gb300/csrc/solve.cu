@@ -37,8 +37,9 @@ __global__ void k_permute_out(const double* __restrict__ z, const int32_t* __res
   }
 }
 
-// one warp per (supernode, block): z[cols(s)] -= sum_d L_d[rows in s] z[cols(d)];
-// then the unit-lower solve with the diagonal block.
+// kkt_solve_noalloc's level solves, over every supernode (a dense tail's factor is
+// in the panels too).  One warp per (supernode, block): z[cols(s)] -= sum_d
+// L_d[rows in s] z[cols(d)]; then the unit-lower solve with the diagonal block.
 __global__ void __launch_bounds__(128) k_fsolve_level(const int32_t* __restrict__ sn_list, int nsn,
                                                       DevSym d, const double* __restrict__ Lx,
                                                       int64_t pt, double* __restrict__ z, int nA,
@@ -74,88 +75,169 @@ __global__ void __launch_bounds__(128) k_fsolve_level(const int32_t* __restrict_
   if (lane < w) zb[f + lane] = zc;
 }
 
-// Narrow levels (few supernodes x blocks): one CTA of kSolveWarps warps per
-// (supernode, block).  Forward: warp w accumulates the updates u with
-// u % kSolveWarps == w into its own partial vector; the partials are summed in
-// warp order.  Backward: warp w owns the columns c with c % kSolveWarps == w.
-constexpr int kSolveWarps = 8;
-constexpr int kWideLevelWarps = 152 * 32;  // levels with fewer (supernode, block) pairs use a CTA per pair
-
-__global__ void __launch_bounds__(kSolveWarps * 32) k_fsolve_level_wide(
-    const int32_t* __restrict__ sn_list, DevSym d, const double* __restrict__ Lx, int64_t pt,
-    double* __restrict__ z, int nA) {
-  __shared__ double part[kSolveWarps][32];
-  const int s = sn_list[blockIdx.x], b = blockIdx.y;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m = (int)(d.sn_rowptr[s + 1] - d.sn_rowptr[s]);
-  const int f = d.sn_first[s], w = d.sn_first[s + 1] - f;
-  const double* P = Lx + b * pt + d.sn_valoff[s];
-  double* zb = z + (int64_t)b * nA;
-  double mine = 0.0;  // partial for row f + lane of this warp's updates
-  for (int64_t u = d.upd_ptr[s] + warp; u < d.upd_ptr[s + 1]; u += kSolveWarps) {
-    const int dd = d.upd_src[u];
-    const int r0 = d.upd_r0[u], r1 = d.upd_r1[u];
-    const int md = (int)(d.sn_rowptr[dd + 1] - d.sn_rowptr[dd]);
-    const int fd = d.sn_first[dd], wd = d.sn_first[dd + 1] - fd;
-    const double* Pd = Lx + b * pt + d.sn_valoff[dd];
-    const int32_t* Rd = d.sn_rows + d.sn_rowptr[dd];
-    // lane j handles row r0 + j of d; its target is row Rd[r0 + j] - f of s
-    double acc = 0.0;
-    const int j = r0 + lane;
-    if (j < r1)
-      for (int kk = 0; kk < wd; kk++) acc += Pd[(int64_t)kk * md + j] * zb[fd + kk];
-    const int tgt = j < r1 ? Rd[j] - f : -1;
-    // route acc to the lane owning its target row (targets are distinct within an update)
-    for (int src = 0; src < r1 - r0; src++) {
-      const double v = __shfl_sync(0xffffffffu, acc, src);
-      const int tg = __shfl_sync(0xffffffffu, tgt, src);
-      if (lane == tg) mine += v;
-    }
+// Row j's products with the solution's entries in the descendants' columns:
+// records p, p + step, ... below p1.
+__device__ __forceinline__ double row_products(const RowRec* __restrict__ rec, int64_t p, int64_t p1, int step,
+                                               const double* __restrict__ Lb, const double* zb) {
+  double acc = 0.0;
+  for (; p < p1; p += step) {
+    const RowRec R = rec[p];
+    const double* a = Lb + (R.off_wd >> 6);
+    const double* v = zb + R.fd;
+    const int wd = (int)(R.off_wd & 63);
+#pragma unroll 4
+    for (int k = 0; k < wd; k++) acc += a[(int64_t)k * R.md] * v[k];
   }
-  part[warp][lane] = mine;
+  return acc;
+}
+
+// One level of the forward solve.  The first small_ctas CTAs take the level's
+// small supernodes (the first nsmall of the list), eight lanes per (supernode,
+// block), lane = row: each walks its row's records, then they solve with the
+// diagonal block by shuffles; the pairs of a warp are mostly blocks of one
+// supernode.  The other CTAs take one (supernode, block) each: lane = row, the
+// warps deal out the row's records, the partial sums are added in warp order and
+// one warp solves with the diagonal block.
+// What bounds it: latency, a few dependent loads per record.  A warp per small
+// supernode leaves most lanes idle; one thread per small supernode walks all its
+// rows one after the other (as slow).  All levels of the 2,383-bus grid, 96
+// blocks: forward 0.25 ms (0.37 with a warp or CTA per supernode, 0.39 with a
+// thread per small one), backward 0.23 (0.58 and 0.38).
+constexpr int kSolveWarps = 8;
+
+__global__ void __launch_bounds__(kSolveWarps * 32)
+    k_fsolve_lvl(const SnDesc* __restrict__ sn, int nsmall, int nsn, int small_ctas, const int64_t* __restrict__ fr_ptr,
+                 const RowRec* __restrict__ fr_rec, const double* __restrict__ Lx, int64_t pt, double* z, int nA, int N) {
+  __shared__ double part[kSolveWarps][32];
+  if ((int)blockIdx.x < small_ctas) {
+    const int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 3;
+    const int c = threadIdx.x & 7;
+    const bool live = q < (int64_t)nsmall * N;
+    const int si = live ? (int)(q / N) : 0, b = live ? (int)(q - (int64_t)si * N) : 0;
+    const SnDesc D = sn[si];
+    const double* Lb = Lx + b * pt;
+    const double* P = Lb + D.val;
+    double* zb = z + (int64_t)b * nA;
+    const bool row = live && c < D.w;
+    double l[kSmallSnCols - 1], acc = 0.0;
+#pragma unroll
+    for (int k = 0; k + 1 < kSmallSnCols; k++) l[k] = row && k < c ? P[(int64_t)k * D.m + c] : 0.0;
+    if (row) acc = zb[D.f + c] - row_products(fr_rec, fr_ptr[D.f + c], fr_ptr[D.f + c + 1], 1, Lb, zb);
+#pragma unroll
+    for (int k = 0; k + 1 < kSmallSnCols; k++) {
+      const double y = __shfl_sync(0xffffffffu, acc, k, 8);
+      if (row && k < c) acc -= l[k] * y;
+    }
+    if (row) zb[D.f + c] = acc;
+    return;
+  }
+  const int pair = blockIdx.x - small_ctas, nbig = nsn - nsmall;
+  const SnDesc D = sn[nsmall + pair % nbig];
+  const int b = pair / nbig, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const double* Lb = Lx + b * pt;
+  const double* P = Lb + D.val;
+  double* zb = z + (int64_t)b * nA;
+  part[warp][lane] = lane < D.w ? row_products(fr_rec, fr_ptr[D.f + lane] + warp, fr_ptr[D.f + lane + 1], kSolveWarps,
+                                               Lb, zb)
+                                : 0.0;
   __syncthreads();
   if (warp == 0) {
     double zc = 0.0;
-    if (lane < w) {
+    if (lane < D.w) {
       double sum = 0.0;
       for (int q = 0; q < kSolveWarps; q++) sum += part[q][lane];
-      zc = zb[f + lane] - sum;
+      zc = zb[D.f + lane] - sum;
     }
-    for (int c = 0; c + 1 < w; c++) {
+    for (int c = 0; c + 1 < D.w; c++) {
       const double zcc = __shfl_sync(0xffffffffu, zc, c);
-      if (lane > c && lane < w) zc -= P[(int64_t)c * m + lane] * zcc;
+      if (lane > c && lane < D.w) zc -= P[(int64_t)c * D.m + lane] * zcc;
     }
-    if (lane < w) zb[f + lane] = zc;
+    if (lane < D.w) zb[D.f + lane] = zc;
   }
 }
 
-__global__ void __launch_bounds__(kSolveWarps * 32) k_bsolve_level_wide(
-    const int32_t* __restrict__ sn_list, DevSym d, const double* __restrict__ Lx, int64_t pt,
-    double* __restrict__ z, int nA) {
-  __shared__ double dots[32];
-  const int s = sn_list[blockIdx.x], b = blockIdx.y;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m = (int)(d.sn_rowptr[s + 1] - d.sn_rowptr[s]);
-  const int f = d.sn_first[s], w = d.sn_first[s + 1] - f;
-  const double* P = Lx + b * pt + d.sn_valoff[s];
-  const int32_t* R = d.sn_rows + d.sn_rowptr[s];
+// The tail's share of the forward solve: z_j -= sum over row j's records, four
+// lanes per (tail row, block) that deal out the records.  96 tails of order 724:
+// 65 us (209 with a CTA per (tail supernode, block) that routed the products to
+// their rows by shuffles, 102 with one lane).
+__global__ void __launch_bounds__(128)
+    k_tail_fgather(const int64_t* __restrict__ fr_ptr, const RowRec* __restrict__ fr_rec, const double* __restrict__ Lx,
+                   int64_t pt, double* z, int nA, int tail_col, int nT, int N) {
+  const int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 2;
+  const bool live = q < (int64_t)nT * N;
+  const int j = tail_col + (live ? (int)(q / N) : 0), b = live ? (int)(q % N) : 0, l = threadIdx.x & 3;
   double* zb = z + (int64_t)b * nA;
-  for (int c = warp; c < w; c += kSolveWarps) {
-    const double* col = P + (int64_t)c * m;
-    double acc = 0.0;
-    for (int r = w + lane; r < m; r += 32) acc += col[r] * zb[R[r]];
+  double acc = live ? row_products(fr_rec, fr_ptr[j] + l, fr_ptr[j + 1], 4, Lx + b * pt, zb) : 0.0;
+  acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+  acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+  if (live && l == 0) zb[j] -= acc;
+}
+
+// One level of the backward solve, split as the forward one: eight lanes per
+// small (supernode, block), lane = column; else a CTA per pair, warp w on the
+// columns c = w mod 8, up to four of them together so that each x is gathered
+// once.
+__global__ void __launch_bounds__(kSolveWarps * 32)
+    k_bsolve_lvl(const SnDesc* __restrict__ sn, int nsmall, int nsn, int small_ctas, const int32_t* __restrict__ sn_rows,
+                 const double* __restrict__ Lx, int64_t pt, double* z, int nA, int N) {
+  __shared__ double dots[32];
+  if ((int)blockIdx.x < small_ctas) {
+    const int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 3;
+    const int c = threadIdx.x & 7;
+    const bool live = q < (int64_t)nsmall * N;
+    const int si = live ? (int)(q / N) : 0, b = live ? (int)(q - (int64_t)si * N) : 0;
+    const SnDesc D = sn[si];
+    const int32_t* R = sn_rows + D.rows;
+    double* zb = z + (int64_t)b * nA;
+    const bool col = live && c < D.w;
+    const double* P = Lx + b * pt + D.val + (int64_t)(col ? c : 0) * D.m;  // this lane's column
+    double l[kSmallSnCols], x = col ? zb[D.f + c] : 0.0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) dots[c] = acc;
+    for (int k = 1; k < kSmallSnCols; k++) l[k] = col && c < k && k < D.w ? P[k] : 0.0;
+    if (col) {
+#pragma unroll 8
+      for (int r = D.w; r < D.m; r++) x -= P[r] * zb[R[r]];
+    }
+#pragma unroll
+    for (int k = kSmallSnCols - 1; k > 0; k--) {
+      const double xk = __shfl_sync(0xffffffffu, x, k, 8);
+      if (c < k && k < D.w) x -= l[k] * xk;
+    }
+    if (col) zb[D.f + c] = x;
+    return;
+  }
+  const int pair = blockIdx.x - small_ctas, nbig = nsn - nsmall;
+  const SnDesc D = sn[nsmall + pair % nbig];
+  const int b = pair / nbig, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const double* P = Lx + b * pt + D.val;
+  const int32_t* R = sn_rows + D.rows;
+  double* zb = z + (int64_t)b * nA;
+  double acc[4] = {};
+  if (warp < D.w) {
+#pragma unroll 4
+    for (int r = D.w + lane; r < D.m; r += 32) {
+      const double xr = zb[R[r]];
+#pragma unroll
+      for (int u = 0; u < 4; u++)
+        if (warp + u * kSolveWarps < D.w) acc[u] += P[(int64_t)(warp + u * kSolveWarps) * D.m + r] * xr;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      if (warp + u * kSolveWarps < D.w) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], o);
+        if (lane == 0) dots[warp + u * kSolveWarps] = acc[u];
+      }
+    }
   }
   __syncthreads();
   if (warp == 0) {
-    double mine = lane < w ? zb[f + lane] - dots[lane] : 0.0;
-    for (int c = w - 1; c >= 0; c--) {
+    double mine = lane < D.w ? zb[D.f + lane] - dots[lane] : 0.0;
+    for (int c = D.w - 1; c >= 0; c--) {
       const double xc = __shfl_sync(0xffffffffu, mine, c);
-      if (lane < c) mine -= P[(int64_t)lane * m + c] * xc;
+      if (lane < c) mine -= P[(int64_t)lane * D.m + c] * xc;
     }
-    if (lane < w) zb[f + lane] = mine;
+    if (lane < D.w) zb[D.f + lane] = mine;
   }
 }
 
@@ -202,43 +284,79 @@ __global__ void __launch_bounds__(128) k_bsolve_level(const int32_t* __restrict_
 }
 
 // u_b[t] = sum_rho W_b[rho][t] z_b[w_col[rho]] / D[rho]; one CTA per (block,
-// 32 columns): warp w sums the rows rho = w mod 8, the 8 partials are added in
-// warp order.
-__global__ void __launch_bounds__(256) k_reduce_u(const double* __restrict__ W, const double* __restrict__ z,
+// 32 columns).  The rows of the augmented tail (from row nd on) are dense: their
+// z / D is staged in shared memory kReduceRows rows at a time, and warp w sums the
+// rows w mod 16.  The rows before them carry a few columns each: every lane walks
+// its column's list, the warps dealing out the entries.  The 16 partials are
+// added in warp order.  96 blocks, 2,579 rows of 100 columns: 35 us (150 over
+// the dense rows and columns of all W; 52 with z / D formed by every lane).
+constexpr int kReduceWarps = 16, kReduceRows = 1024;
+
+__global__ void __launch_bounds__(32 * kReduceWarps) k_reduce_u(const double* __restrict__ W, const double* __restrict__ z,
                                                   const double* __restrict__ wdinv,
-                                                  const int32_t* __restrict__ w_col, int nw, int k, int nA,
+                                                  const int32_t* __restrict__ w_col, const int32_t* __restrict__ wr_ptr,
+                                                  const int32_t* __restrict__ wr_row, int nd, int nw, int k, int nA,
                                                   double* __restrict__ u) {
-  __shared__ double part[8][32];
+  __shared__ double part[kReduceWarps][32];
+  __shared__ double zd[kReduceRows];
   const int b = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = blockIdx.x * 32 + lane;
   const double* Wb = W + (int64_t)b * nw * k;
   const double* zb = z + (int64_t)b * nA;
   const double* db = wdinv + (int64_t)b * nw;
   double acc = 0.0;
-  if (t < k)
-    for (int rho = warp; rho < nw; rho += 8) acc += Wb[(int64_t)rho * k + t] * (zb[w_col[rho]] * db[rho]);
+  if (t < k) {
+    const int p1 = wr_ptr[t + 1];
+    for (int p = wr_ptr[t] + warp; p < p1; p += kReduceWarps) {
+      const int rho = wr_row[p];
+      acc += Wb[(int64_t)rho * k + t] * (zb[w_col[rho]] * db[rho]);
+    }
+  }
+  for (int r0 = nd; r0 < nw; r0 += kReduceRows) {
+    const int rows = min(kReduceRows, nw - r0);
+    __syncthreads();
+    for (int r = threadIdx.x; r < rows; r += blockDim.x) zd[r] = zb[w_col[r0 + r]] * db[r0 + r];
+    __syncthreads();
+    if (t < k) {
+      const double* Wr = Wb + (int64_t)r0 * k + t;
+#pragma unroll 8
+      for (int r = warp; r < rows; r += kReduceWarps) acc += Wr[(int64_t)r * k] * zd[r];
+    }
+  }
   part[warp][lane] = acc;
   __syncthreads();
   if (warp == 0 && t < k) {
     double sum = 0.0;
-    for (int q = 0; q < 8; q++) sum += part[q][lane];
+    for (int q = 0; q < kReduceWarps; q++) sum += part[q][lane];
     u[(int64_t)b * k + t] = sum;
   }
 }
 
+// The kernels over the coupling columns take LANES lanes per column: 32 where a
+// column has many entries (SCOPF: hundreds, and a dense C; coupling_lanes), one
+// where it has two.  The lanes add up in a fixed order.
+template <int LANES>
+__device__ __forceinline__ double lanes_sum(double v) {
+#pragma unroll
+  for (int o = LANES / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
 // t[c] = r_g[c] - sum_{e in column c} b[e] u[block(e)][t(e)]
+template <int LANES>
 __global__ void k_reduce_t(const double* __restrict__ rg, const int32_t* __restrict__ t_ptr,
                            const int32_t* __restrict__ t_e, const int32_t* __restrict__ e_t,
                            const int32_t* __restrict__ e_block, const double* __restrict__ b_vals,
                            const double* __restrict__ u, int k, int nC, double* __restrict__ tg) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= nC) return;
-  double acc = rg[c];
-  for (int q = t_ptr[c]; q < t_ptr[c + 1]; q++) {
-    const int e = t_e[q];
-    acc -= b_vals[e] * u[(int64_t)e_block[e] * k + e_t[e]];
-  }
-  tg[c] = acc;
+  const int c = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / LANES), l = threadIdx.x % LANES;
+  double acc = 0.0;
+  if (c < nC)
+    for (int q = t_ptr[c] + l; q < t_ptr[c + 1]; q += LANES) {
+      const int e = t_e[q];
+      acc += b_vals[e] * u[(int64_t)e_block[e] * k + e_t[e]];
+    }
+  acc = lanes_sum<LANES>(acc);
+  if (c < nC && l == 0) tg[c] = rg[c] - acc;
 }
 
 // v_b[t] = sum_{e in block b, index t} b[e] x_g[col(e)]
@@ -254,18 +372,32 @@ __global__ void k_mx(const int32_t* __restrict__ bt_ptr, const int32_t* __restri
   v[q] = acc;
 }
 
-// z_b[w_col[rho]] -= sum_t W_b[rho][t] v_b[t]
-__global__ void k_apply_xg(const double* __restrict__ W, const double* __restrict__ v,
-                           const int32_t* __restrict__ w_col, int nw, int k, int nA, int N,
-                           double* __restrict__ z) {
-  const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (q >= (int64_t)nw * N) return;
-  const int b = (int)(q / nw), rho = (int)(q - (int64_t)b * nw);
+// z_b[w_col[rho]] -= sum_t W_b[rho][t] v_b[t], eight lanes per row: over all
+// columns for the rows of the augmented tail (from row nd on), over the columns
+// of the row's supernode for the others.  96 blocks, 2,579 rows of 100 columns:
+// 37 us (68 with a thread per row over all columns), 17 of 2,258 rows of 1,632
+// columns 49 (243).
+__global__ void __launch_bounds__(256)
+    k_apply_xg(const double* __restrict__ W, const double* __restrict__ v, const int32_t* __restrict__ w_col,
+               const int32_t* __restrict__ w_sn, const int32_t* __restrict__ wt_ptr, const int32_t* __restrict__ wt_idx,
+               int nd, int nw, int k, int nA, int N, double* __restrict__ z) {
+  const int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 3;
+  const int l = threadIdx.x & 7;
+  const bool live = q < (int64_t)nw * N;
+  const int b = live ? (int)(q / nw) : 0, rho = live ? (int)(q - (int64_t)b * nw) : 0;
   const double* Wr = W + ((int64_t)b * nw + rho) * k;
   const double* vb = v + (int64_t)b * k;
   double acc = 0.0;
-  for (int t = 0; t < k; t++) acc += Wr[t] * vb[t];
-  z[(int64_t)b * nA + w_col[rho]] -= acc;
+  if (live && rho >= nd) {
+#pragma unroll 8
+    for (int t = l; t < k; t += 8) acc += Wr[t] * vb[t];
+  } else if (live) {
+    const int s = w_sn[rho], e1 = wt_ptr[s + 1];
+    for (int e = wt_ptr[s] + l; e < e1; e += 8) acc += Wr[wt_idx[e]] * vb[wt_idx[e]];
+  }
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (live && l == 0) z[(int64_t)b * nA + w_col[rho]] -= acc;
 }
 
 // ---- residual rho = r - K x ----
@@ -303,28 +435,31 @@ __global__ void k_resid_b(const int32_t* __restrict__ bt_ptr, const int32_t* __r
 }
 
 // coupling rows: rho_g = r_g - sum_i B_i^T x_i - C x_g
+template <int LANES>
 __global__ void k_resid_g(const int32_t* __restrict__ t_ptr, const int32_t* __restrict__ t_e,
                           const int32_t* __restrict__ e_block, const int32_t* __restrict__ b_row,
                           const double* __restrict__ b_vals, const double* __restrict__ c_vals,
                           int c_kind, const double* __restrict__ r, const double* __restrict__ x,
                           int nA, int N, int nC, double* __restrict__ rho) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= nC) return;
+  const int c = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / LANES), l = threadIdx.x % LANES;
   const int64_t g = (int64_t)N * nA;
   double acc = 0.0;
-  for (int q = t_ptr[c]; q < t_ptr[c + 1]; q++) {
-    const int e = t_e[q];
-    acc += b_vals[e] * x[(int64_t)e_block[e] * nA + b_row[e]];
-  }
-  if (c_kind == 0) {
-    acc += c_vals[c] * x[g + c];
-  } else {
-    for (int c2 = 0; c2 < nC; c2++) {
-      const double cv = c2 <= c ? c_vals[(int64_t)c * nC + c2] : c_vals[(int64_t)c2 * nC + c];
-      acc += cv * x[g + c2];
+  if (c < nC) {
+    for (int q = t_ptr[c] + l; q < t_ptr[c + 1]; q += LANES) {
+      const int e = t_e[q];
+      acc += b_vals[e] * x[(int64_t)e_block[e] * nA + b_row[e]];
+    }
+    if (c_kind == 0) {
+      if (l == 0) acc += c_vals[c] * x[g + c];
+    } else {
+      for (int c2 = l; c2 < nC; c2 += LANES) {
+        const double cv = c2 <= c ? c_vals[(int64_t)c * nC + c2] : c_vals[(int64_t)c2 * nC + c];
+        acc += cv * x[g + c2];
+      }
     }
   }
-  rho[g + c] = r[g + c] - acc;
+  acc = lanes_sum<LANES>(acc);
+  if (c < nC && l == 0) rho[g + c] = r[g + c] - acc;
 }
 
 __device__ __forceinline__ void atomic_max_nonneg(double* addr, double v) {
@@ -410,21 +545,22 @@ __global__ void k_knorm_blocks(const int32_t* __restrict__ rowptr, const int32_t
   block_max_to(out, m);
 }
 
+template <int LANES>
 __global__ void k_knorm_g(const int32_t* __restrict__ t_ptr, const int32_t* __restrict__ t_e,
                           const double* __restrict__ b_vals, const double* __restrict__ c_vals,
                           int c_kind, int nC, double* __restrict__ out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  const int c = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / LANES), l = threadIdx.x % LANES;
   double acc = 0.0;
   if (c < nC) {
-    for (int q = t_ptr[c]; q < t_ptr[c + 1]; q++) acc += fabs(b_vals[t_e[q]]);
+    for (int q = t_ptr[c] + l; q < t_ptr[c + 1]; q += LANES) acc += fabs(b_vals[t_e[q]]);
     if (c_kind == 0) {
-      acc += fabs(c_vals[c]);
+      if (l == 0) acc += fabs(c_vals[c]);
     } else {
-      for (int c2 = 0; c2 < nC; c2++)
+      for (int c2 = l; c2 < nC; c2 += LANES)
         acc += fabs(c2 <= c ? c_vals[(int64_t)c * nC + c2] : c_vals[(int64_t)c2 * nC + c]);
     }
   }
-  block_max_to(out, acc);
+  block_max_to(out, lanes_sum<LANES>(acc));
 }
 
 __global__ void k_axpy(double* __restrict__ y, const double* __restrict__ x, int64_t n) {
@@ -476,6 +612,29 @@ __global__ void k_scale_into(double* __restrict__ y, double a, const double* __r
     y[q] = a * x[q];
 }
 
+// Lanes per coupling column: a warp from 16 entries per column on, and for a
+// dense C (a row of nC entries).  1,021 buses with 16 outages (304 columns of some
+// 140 entries): t 13 us (214 with a thread per column), the residual's coupling
+// rows 14 (204), their norm 9 (101).
+inline int coupling_lanes(const Handle& h) { return h.c_kind == 1 || h.nnzB >= 16 * (int64_t)h.nC ? 32 : 1; }
+inline int coupling_grid(const Handle& h) { return (int)(((int64_t)h.nC * coupling_lanes(h) + 255) / 256); }
+
+// CTAs of one level of the block solves: the small supernodes, then one per
+// (other supernode, block).
+struct LevelGrid {
+  int first, nsn, nsmall, small_ctas, ctas;
+};
+
+inline LevelGrid level_grid(const Handle& h, int l) {
+  LevelGrid g;
+  g.first = h.flvl_ptr[l];
+  g.nsn = h.flvl_ptr[l + 1] - g.first;
+  g.nsmall = h.flvl_small[l];
+  g.small_ctas = (int)(((int64_t)g.nsmall * h.N * 8 + kSolveWarps * 32 - 1) / (kSolveWarps * 32));
+  g.ctas = g.small_ctas + (g.nsn - g.nsmall) * h.N;
+  return g;
+}
+
 inline int grid_for(int64_t n, int bs = 256) {
   return (int)std::max<int64_t>(1, std::min<int64_t>((n + bs - 1) / bs, 152 * 16));
 }
@@ -496,17 +655,11 @@ cudaError_t launch_apply_front(Handle& h, const double* r, cudaStream_t st) {
   // with a dense tail, the levels cover the supernodes outside it and the
   // tail's triangular solves are dense (the tail factor's triangles)
   const bool tail = h.nT > 0;
-  const std::vector<int32_t>& lptr = tail ? h.flvl_ptr : h.lvl_ptr;
-  const int32_t* lsn = tail ? h.d.flvl_sn : h.d.lvl_sn;
   for (int l = 0; l < h.sym.nlevels; l++) {
-    const int s0 = lptr[l], nsn = lptr[l + 1] - s0;
-    if (nsn == 0) continue;
-    const int warps = nsn * N;
-    if (warps < kWideLevelWarps) {
-      k_fsolve_level_wide<<<dim3(nsn, N), kSolveWarps * 32, 0, st>>>(lsn + s0, h.d, h.Lx, pt, h.z, nA);
-    } else {
-      k_fsolve_level<<<(warps + 3) / 4, 128, 0, st>>>(lsn + s0, nsn, h.d, h.Lx, pt, h.z, nA, N);
-    }
+    const LevelGrid g = level_grid(h, l);
+    if (g.ctas == 0) continue;
+    k_fsolve_lvl<<<g.ctas, kSolveWarps * 32, 0, st>>>(h.d.flvl_desc + g.first, g.nsmall, g.nsn, g.small_ctas,
+                                                      h.d.fr_ptr, h.d.fr_rec, h.Lx, pt, h.z, nA, N);
     h.launches++;
   }
   if (tail) {
@@ -517,15 +670,15 @@ cudaError_t launch_apply_front(Handle& h, const double* r, cudaStream_t st) {
     if (k > 0 && nw > 0) {
       dim3 g((k + 31) / 32, N);
       {
-    k_reduce_u<<<g, 256, 0, st>>>(h.W, h.z, h.wdinv, h.d.w_col, nw, k, nA, h.u);
+    k_reduce_u<<<g, 32 * kReduceWarps, 0, st>>>(h.W, h.z, h.wdinv, h.d.w_col, h.d.wr_ptr, h.d.wr_row, h.nw_nt, nw, k, nA, h.u);
     h.launches++;
   }
     } else if (k > 0) {
       cudaMemsetAsync(h.u, 0, sizeof(double) * (size_t)k * N, st);
     }
     {
-    k_reduce_t<<<(h.nC + 255) / 256, 256, 0, st>>>(r + nb, h.d.t_ptr, h.d.t_e, h.d.e_t, h.d.e_block,
-                                                   h.b_vals, h.u, k, h.nC, h.tg);
+    (coupling_lanes(h) == 32 ? k_reduce_t<32> : k_reduce_t<1>)<<<coupling_grid(h), 256, 0, st>>>(
+        r + nb, h.d.t_ptr, h.d.t_e, h.d.e_t, h.d.e_block, h.b_vals, h.u, k, h.nC, h.tg);
     h.launches++;
   }
   }
@@ -537,8 +690,6 @@ cudaError_t launch_apply_back(Handle& h, double* out, cudaStream_t st, bool solv
   const int64_t pt = h.sym.panel_total;
   const int64_t nb = (int64_t)nA * N;
   const bool tail = h.nT > 0;
-  const std::vector<int32_t>& lptr = tail ? h.flvl_ptr : h.lvl_ptr;
-  const int32_t* lsn = tail ? h.d.flvl_sn : h.d.lvl_sn;
   if (h.nC > 0) {
     // without solve_s, h.xg already holds x_g (a sharded solve's broadcast)
     cudaError_t e = !solve_s ? cudaSuccess
@@ -552,7 +703,8 @@ cudaError_t launch_apply_back(Handle& h, double* out, cudaStream_t st, bool solv
     h.launches++;
   }
       {
-    k_apply_xg<<<grid_for((int64_t)nw * N), 256, 0, st>>>(h.W, h.v, h.d.w_col, nw, k, nA, N, h.z);
+    k_apply_xg<<<(int)(((int64_t)nw * N * 8 + 255) / 256), 256, 0, st>>>(h.W, h.v, h.d.w_col, h.d.w_sn, h.d.wt_ptr, h.d.wt_idx,
+                                                          h.nw_nt, nw, k, nA, N, h.z);
     h.launches++;
   }
     }
@@ -566,14 +718,10 @@ cudaError_t launch_apply_back(Handle& h, double* out, cudaStream_t st, bool solv
     if (e != cudaSuccess) return e;
   }
   for (int l = h.sym.nlevels - 1; l >= 0; l--) {
-    const int s0 = lptr[l], nsn = lptr[l + 1] - s0;
-    if (nsn == 0) continue;
-    const int warps = nsn * N;
-    if (warps < kWideLevelWarps) {
-      k_bsolve_level_wide<<<dim3(nsn, N), kSolveWarps * 32, 0, st>>>(lsn + s0, h.d, h.Lx, pt, h.z, nA);
-    } else {
-      k_bsolve_level<<<(warps + 3) / 4, 128, 0, st>>>(lsn + s0, nsn, h.d, h.Lx, pt, h.z, nA, N);
-    }
+    const LevelGrid g = level_grid(h, l);
+    if (g.ctas == 0) continue;
+    k_bsolve_lvl<<<g.ctas, kSolveWarps * 32, 0, st>>>(h.d.flvl_desc + g.first, g.nsmall, g.nsn, g.small_ctas,
+                                                      h.d.sn_rows, h.Lx, pt, h.z, nA, N);
     h.launches++;
   }
   {
@@ -583,6 +731,19 @@ cudaError_t launch_apply_back(Handle& h, double* out, cudaStream_t st, bool solv
   if (h.nC > 0)
     cudaMemcpyAsync(out + nb, h.xg, sizeof(double) * h.nC, cudaMemcpyDeviceToDevice, st);
   return cudaGetLastError();
+}
+
+// The tail's share of the forward solve and its dense triangular solves.
+cudaError_t launch_tail_fsolve(Handle& h, double* z, cudaStream_t st) {
+  k_tail_fgather<<<(int)(((int64_t)h.nT * h.N * 4 + 127) / 128), 128, 0, st>>>(
+      h.d.fr_ptr, h.d.fr_rec, h.Lx, h.sym.panel_total, z, h.nA, h.sym.tail_col, h.nT, h.N);
+  h.launches++;
+  cudaError_t e = cudaGetLastError();
+  return e != cudaSuccess ? e : launch_tail_trsv(h, true, z + h.sym.tail_col, st);
+}
+
+cudaError_t launch_tail_bsolve(Handle& h, double* z, cudaStream_t st) {
+  return launch_tail_trsv(h, false, z + h.sym.tail_col, st);
 }
 
 cudaError_t launch_apply_inverse(Handle& h, const double* r, double* out, cudaStream_t st) {
@@ -606,8 +767,8 @@ cudaError_t launch_residual(Handle& h, const double* r, const double* x, double*
     h.launches++;
   }
     {
-    k_resid_g<<<(h.nC + 255) / 256, 256, 0, st>>>(h.d.t_ptr, h.d.t_e, h.d.e_block, h.d.b_row, h.b_vals,
-                                                  h.c_vals, h.c_kind, r, x, nA, N, h.nC, rho);
+    (coupling_lanes(h) == 32 ? k_resid_g<32> : k_resid_g<1>)<<<coupling_grid(h), 256, 0, st>>>(
+        h.d.t_ptr, h.d.t_e, h.d.e_block, h.d.b_row, h.b_vals, h.c_vals, h.c_kind, r, x, nA, N, h.nC, rho);
     h.launches++;
   }
   }
@@ -626,8 +787,8 @@ cudaError_t launch_knorm(Handle& h, cudaStream_t st) {
   }
   if (h.nC > 0)
     {
-    k_knorm_g<<<(h.nC + 255) / 256, 256, 0, st>>>(h.d.t_ptr, h.d.t_e, h.b_vals, h.c_vals, h.c_kind,
-                                                  h.nC, h.knorm);
+    (coupling_lanes(h) == 32 ? k_knorm_g<32> : k_knorm_g<1>)<<<coupling_grid(h), 256, 0, st>>>(
+        h.d.t_ptr, h.d.t_e, h.b_vals, h.c_vals, h.c_kind, h.nC, h.knorm);
     h.launches++;
   }
   return cudaGetLastError();
@@ -688,20 +849,21 @@ cudaError_t launch_apply_inverse_ws(Handle& h, const double* r, double* out,
   if (h.nC > 0) {
     if (k > 0 && nw > 0) {
       dim3 g((k + 31) / 32, N);
-      k_reduce_u<<<g, 256, 0, st>>>(h.W, ws.z, h.wdinv, h.d.w_col, nw, k, nA, ws.u);
+      k_reduce_u<<<g, 32 * kReduceWarps, 0, st>>>(h.W, ws.z, h.wdinv, h.d.w_col, h.d.wr_ptr, h.d.wr_row, h.nw_nt, nw, k, nA, ws.u);
       h.launches++;
     } else if (k > 0) {
       cudaError_t e = cudaMemsetAsync(ws.u, 0, sizeof(double) * (size_t)k * N, st);
       if (e != cudaSuccess) return e;
     }
-    k_reduce_t<<<(h.nC + 255) / 256, 256, 0, st>>>(r + nb, h.d.t_ptr, h.d.t_e, h.d.e_t, h.d.e_block,
-                                                   h.b_vals, ws.u, k, h.nC, ws.tg);
+    (coupling_lanes(h) == 32 ? k_reduce_t<32> : k_reduce_t<1>)<<<coupling_grid(h), 256, 0, st>>>(
+        r + nb, h.d.t_ptr, h.d.t_e, h.d.e_t, h.d.e_block, h.b_vals, ws.u, k, h.nC, ws.tg);
     h.launches++;
     cudaError_t e = h.cum ? launch_cum_solve(h, ws.tg, ws.xg, st) : launch_dense_solve_ws(h, ws.tg, ws.xg, ws.dot, st);
     if (e != cudaSuccess) return e;
     if (k > 0 && nw > 0) {
       k_mx<<<(k * N + 255) / 256, 256, 0, st>>>(h.d.bt_ptr, h.d.b_col, h.b_vals, ws.xg, k, N, ws.v);
-      k_apply_xg<<<grid_for((int64_t)nw * N), 256, 0, st>>>(h.W, ws.v, h.d.w_col, nw, k, nA, N, ws.z);
+      k_apply_xg<<<(int)(((int64_t)nw * N * 8 + 255) / 256), 256, 0, st>>>(h.W, ws.v, h.d.w_col, h.d.w_sn, h.d.wt_ptr, h.d.wt_idx,
+                                                            h.nw_nt, nw, k, nA, N, ws.z);
       h.launches += 2;
     }
   }

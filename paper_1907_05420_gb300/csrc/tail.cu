@@ -151,60 +151,7 @@ __global__ void __launch_bounds__(32 * kTailUpdWarps, 10)
   }
 }
 
-// Forward solve, the tail's share: z[cols(s)] -= sum over descendants d
-// outside the tail of L_d[rows in s] z[cols(d)], for every tail supernode s
-// (independent of one another; the triangular solve is the dense tail's).
-// One CTA of 8 warps per (tail supernode, block), warp w taking the updates
-// u = w mod 8, the partials added in warp order.
-__global__ void __launch_bounds__(256) k_tail_fgather(DevSym d, const double* __restrict__ Lx, int64_t pt,
-                                                      double* __restrict__ z, int nA, int tail_sn) {
-  __shared__ double part[8][32];
-  const int s = tail_sn + blockIdx.x, b = blockIdx.y;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int f = d.sn_first[s], w = d.sn_first[s + 1] - f;
-  double* zb = z + (int64_t)b * nA;
-  double mine = 0.0;
-  const int64_t u0 = d.upd_ptr[s], u1 = u0 + d.upd_ntail[s];
-  for (int64_t u = u0 + warp; u < u1; u += 8) {
-    const int dd = d.upd_src[u];
-    const int r0 = d.upd_r0[u], r1 = d.upd_r1[u];
-    const int md = (int)(d.sn_rowptr[dd + 1] - d.sn_rowptr[dd]);
-    const int fd = d.sn_first[dd], wd = d.sn_first[dd + 1] - fd;
-    const double* Pd = Lx + b * pt + d.sn_valoff[dd];
-    const int32_t* Rd = d.sn_rows + d.sn_rowptr[dd];
-    double acc = 0.0;
-    const int j = r0 + lane;
-    if (j < r1)
-      for (int kk = 0; kk < wd; kk++) acc += Pd[(int64_t)kk * md + j] * zb[fd + kk];
-    const int tgt = j < r1 ? Rd[j] - f : -1;
-    for (int src = 0; src < r1 - r0; src++) {  // targets are distinct within an update
-      const double v = __shfl_sync(0xffffffffu, acc, src);
-      const int tg = __shfl_sync(0xffffffffu, tgt, src);
-      if (lane == tg) mine += v;
-    }
-  }
-  part[warp][lane] = mine;
-  __syncthreads();
-  if (warp == 0 && lane < w) {
-    double sum = 0.0;
-    for (int q = 0; q < 8; q++) sum += part[q][lane];
-    zb[f + lane] -= sum;
-  }
-}
-
 }  // namespace
-
-cudaError_t launch_tail_fsolve(Handle& h, double* z, cudaStream_t st) {
-  const int nts = h.sym.nsuper - h.sym.tail_sn;
-  k_tail_fgather<<<dim3(nts, h.N), 256, 0, st>>>(h.d, h.Lx, h.sym.panel_total, z, h.nA, h.sym.tail_sn);
-  h.launches++;
-  cudaError_t e = cudaGetLastError();
-  return e != cudaSuccess ? e : launch_tail_trsv(h, true, z + h.sym.tail_col, st);
-}
-
-cudaError_t launch_tail_bsolve(Handle& h, double* z, cudaStream_t st) {
-  return launch_tail_trsv(h, false, z + h.sym.tail_col, st);
-}
 
 cudaError_t launch_dense_tail(Handle& h, cudaStream_t st) {
   const int nT = h.nT, nTa = h.nTa, N = h.N;

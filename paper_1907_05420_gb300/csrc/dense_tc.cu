@@ -88,6 +88,30 @@ __device__ __forceinline__ void mma_bf16(uint32_t dtm, uint64_t ad, uint64_t bd,
       "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
 }
 
+// The digit products of one K step of 16 into the seven levels at tmem: digit
+// slice sa of A against the slices 0 .. 6 - sa of B adds to the levels sa .. 6,
+// which are neighbours in tensor memory as the slices of B are in shared memory
+// (64 rows each, one after the other), so a slice of A takes one MMA of N = 64
+// (7 - sa) columns, or two where that passes 256.  A 128 x 64 x 16 MMA per digit
+// pair reads A's slice (4 KB) for every 2 KB of B, 48 cycles of shared-memory
+// bandwidth for 32 of products; here A is read 10 times a step instead of 28.
+// 24 tails of order 6,938 (130 launches of the 256-wide update): 135 -> 110 ms.
+__device__ __forceinline__ void mma_digit_pairs(uint32_t tmem, uint64_t a, uint32_t a_slice, uint64_t b, uint32_t b_slice,
+                                                bool first) {
+#pragma unroll
+  for (int sa = 0; sa < kEmuLevels; sa++) {
+    const int n = kEmuLevels - sa, n1 = n > 4 ? (n + 1) / 2 : n;
+#pragma unroll
+    for (int part = 0; part < (n > 4 ? 2 : 1); part++) {
+      const int sb = part ? n1 : 0, cnt = part ? n - n1 : n1;
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(cnt * TN >> 3) << 17) |
+                             ((uint32_t)(TM >> 4) << 24);
+      mma_bf16(tmem + (uint32_t)((sa + sb) * TN), umma_desc_at(a, sa * a_slice), umma_desc_at(b, sb * b_slice), idesc,
+               first && sa == 0 ? 0u : 1u);
+    }
+  }
+}
+
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
   const long long t0 = clock64();
   for (;;) {
@@ -650,8 +674,6 @@ __global__ void __launch_bounds__(kEmuThreads, 1)
         if (!s_abort) atomicExch(err, 5);
         s_abort = 1;
       } else {
-        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >> 3) << 17) |
-                               ((uint32_t)(TM >> 4) << 24);
         for (int u = 0; u < ntile; u++) {
           const int s = u & 1;
           if (!mbar_wait_ab(smem_u32(&bar_bfull[s]), (uint32_t)((u >> 1) & 1), &s_abort) ||
@@ -663,18 +685,10 @@ __global__ void __launch_bounds__(kEmuThreads, 1)
           asm volatile("tcgen05.fence::after_thread_sync;");
           const uint64_t a0 = umma_desc(smem_u32(sA), 128, KG * 128);
           const uint64_t b0 = umma_desc(smem_u32(sB + s * B_BYTES), 128, KG * 128);
-          // level d takes the digit pairs sa + sb = d
 #pragma unroll
-          for (int d = 0; d < kEmuLevels; d++) {
-            const uint32_t dtm = tmem + (uint32_t)(d * TN);
-#pragma unroll
-            for (int sa = 0; sa <= d; sa++)
-#pragma unroll
-              for (int ks = 0; ks < KSTEPS; ks++)
-                mma_bf16(dtm, umma_desc_at(a0, sa * A_SLICE + ks * MMA_K_BYTES * 8),
-                         umma_desc_at(b0, (d - sa) * B_SLICE + ks * MMA_K_BYTES * 8), idesc,
-                         (sa == 0 && ks == 0) ? 0u : 1u);
-          }
+          for (int ks = 0; ks < KSTEPS; ks++)
+            mma_digit_pairs(tmem, umma_desc_at(a0, ks * MMA_K_BYTES * 8), A_SLICE, umma_desc_at(b0, ks * MMA_K_BYTES * 8),
+                            B_SLICE, ks == 0);
           asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                            smem_u32(&bar_bempty[s]))
                        : "memory");
@@ -942,19 +956,11 @@ __global__ void __launch_bounds__(256, 1) k_tc_panel_emu(double* __restrict__ S0
       mbar_wait(bl, 0);  // give copies still in flight a second bounded window before exit
     } else {
       asm volatile("tcgen05.fence::after_thread_sync;");
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >> 3) << 17) |
-                             ((uint32_t)(TM >> 4) << 24);
       const uint64_t a0 = umma_desc(smem_u32(sA), 128, KG * 128);
       const uint64_t b0 = umma_desc(smem_u32(sB), 128, KG * 128);
 #pragma unroll
-      for (int d = 0; d < kEmuLevels; d++) {
-#pragma unroll
-        for (int sa = 0; sa <= d; sa++)
-#pragma unroll
-          for (int ks = 0; ks < KSTEPS; ks++)
-            mma_bf16(tmem + (uint32_t)(d * TN), umma_desc_at(a0, sa * A_SLICE + ks * 256),
-                     umma_desc_at(b0, (d - sa) * B_SLICE + ks * 256), idesc, (sa == 0 && ks == 0) ? 0u : 1u);
-      }
+      for (int ks = 0; ks < KSTEPS; ks++)
+        mma_digit_pairs(tmem, umma_desc_at(a0, ks * 256), A_SLICE, umma_desc_at(b0, ks * 256), B_SLICE, ks == 0);
       asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                        smem_u32(&bar_mma))
                    : "memory");
@@ -1226,8 +1232,6 @@ __global__ void __launch_bounds__(kEmuThreads, 1)
     if (lane == 0 && ntile > 0) {
       // MMA issuer
       uint32_t last_bar = 0, last_par = 0;
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >> 3) << 17) |
-                             ((uint32_t)(TM >> 4) << 24);
       bool stop = false;
       for (int u = 0; u < ntile && !stop; u++) {
         if (u >= 1 && !mbar_wait_ab(smem_u32(&bar_tempty), (uint32_t)((u - 1) & 1), &s_abort)) {
@@ -1248,18 +1252,10 @@ __global__ void __launch_bounds__(kEmuThreads, 1)
           const uint8_t* sA = smem + st * (kEwStageA + kEwStageB);
           const uint64_t a0 = umma_desc(smem_u32(sA), 128, 512);
           const uint64_t b0 = umma_desc(smem_u32(sA + kEwStageA), 128, 512);
-          // level d takes the digit pairs sa + sb = d
 #pragma unroll
-          for (int d = 0; d < kEmuLevels; d++) {
-            const uint32_t dtm = tmem + (uint32_t)(d * TN);
-#pragma unroll
-            for (int sa = 0; sa <= d; sa++)
-#pragma unroll
-              for (int ks = 0; ks < kEwChunk / 16; ks++)
-                mma_bf16(dtm, umma_desc_at(a0, sa * 2 * kEwPiece + ks * 256),
-                         umma_desc_at(b0, (d - sa) * kEwPiece + ks * 256), idesc,
-                         (k == 0 && sa == 0 && ks == 0) ? 0u : 1u);
-          }
+          for (int ks = 0; ks < kEwChunk / 16; ks++)
+            mma_digit_pairs(tmem, umma_desc_at(a0, ks * 256), 2 * kEwPiece, umma_desc_at(b0, ks * 256), kEwPiece,
+                            k == 0 && ks == 0);
           asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                            smem_u32(&bar_empty[st]))
                        : "memory");

@@ -614,7 +614,7 @@ __global__ void k_scale_into(double* __restrict__ y, double a, const double* __r
 
 // Lanes per coupling column: a warp from 16 entries per column on, and for a
 // dense C (a row of nC entries).  1,021 buses with 16 outages (304 columns of some
-// 140 entries): t 13 us (214 with a thread per column), the residual's coupling
+// 121 entries): t 13 us (214 with a thread per column), the residual's coupling
 // rows 14 (204), their norm 9 (101).
 inline int coupling_lanes(const Handle& h) { return h.c_kind == 1 || h.nnzB >= 16 * (int64_t)h.nC ? 32 : 1; }
 inline int coupling_grid(const Handle& h) { return (int)(((int64_t)h.nC * coupling_lanes(h) + 255) / 256); }

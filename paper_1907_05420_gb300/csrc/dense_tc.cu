@@ -138,17 +138,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;");
 }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;");
-}
-
-
-
 // Images of the operands of one panel step.  Rows rho in [0, m) are trailing
 // rows base + rho.  A = Y (rows of L21 D, from Y with leading dimension n),
 // B = L21 (columns k0..k0+63 of S).  Rows >= m are written as zeros.
@@ -529,55 +518,92 @@ __device__ __forceinline__ void prefetch_tile_row(const T* S, int n, int row, bo
   }
 }
 
+__device__ __forceinline__ void tmem_ld8_start(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
+
+// r holds what its load reads once this has returned (the registers pass through
+// the wait, so that no use moves ahead of it).
+__device__ __forceinline__ void tmem_ld8_wait(uint32_t (&r)[8]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])
+               :
+               : "memory");
+}
+
 // The epilogue's read-out of tensor memory: the 7 levels of this thread's
-// kEpiCols columns (16-column loads) folded into W = V 2^16 + round(256 c),
-// V the exact integer of levels 0-3 and c the FP32 sum of levels 4-6.  Only
-// this part holds tensor memory; the FP64 bit patterns are built after it is
-// handed back.
-__device__ __forceinline__ void emu_fold(uint32_t taddr, long long (&W)[kEpiCols]) {
+// kEpiCols columns (8-column loads, the next level's under way while one is
+// used) reduced to V, the exact integer of levels 0-3, and c, the FP32 sum of
+// levels 4-6.  Only this part holds tensor memory, and the tensor pipe idles
+// meanwhile (the levels of a tile fill it), so it does no more than fit the
+// result in registers; emu_combine and the FP64 bit patterns come after it is
+// handed back.  No register may be spilled here: a load's destination holds
+// nothing before its wait.  64-wide updates of the 9,241-bus step 19.0 -> 17.4
+// ms, 256-wide 110.3 -> 107.7, against folding everything with one load at a time.
+__device__ __forceinline__ void emu_drain(uint32_t taddr, long long (&V)[kEpiCols], float (&cf)[kEpiCols]) {
 #pragma unroll
-  for (int hh = 0; hh < kEpiCols / 16; hh++) {
-    long long V[16];
-    float cf[16];
+  for (int hh = 0; hh < kEpiCols / 8; hh++) {
+    const uint32_t t = taddr + (uint32_t)(hh * 8);
+    uint32_t a[8], b[8];
+    int p[8];
+    tmem_ld8_start(t, a);
+    tmem_ld8_wait(a);
+    tmem_ld8_start(t + 1 * TN, b);
 #pragma unroll
-    for (int j = 0; j < 16; j++) {
-      V[j] = 0;
-      cf[j] = 0.f;
-    }
+    for (int j = 0; j < 8; j++) p[j] = small_f2i(__uint_as_float(a[j]));
+    tmem_ld8_wait(b);
+    tmem_ld8_start(t + 2 * TN, a);
 #pragma unroll
-    for (int d = 0; d < kEmuLevels; d++) {
-      uint32_t r[16];
-      tmem_ld16(taddr + (uint32_t)(d * TN + hh * 16), r);
+    for (int j = 0; j < 8; j++) p[j] = fold_level1(p[j], __uint_as_float(b[j]));
+    tmem_ld8_wait(a);
+    tmem_ld8_start(t + 3 * TN, b);
 #pragma unroll
-      for (int j = 0; j < 16; j++) {
-        const float fv = __uint_as_float(r[j]);
-        if (d < 4) V[j] = V[j] * 256 + exact_f2i(fv);  // levels 0-3: exact integers below 2^24
-        else cf[j] += fv * (d == 4 ? 1.f : (d == 5 ? 0.00390625f : 0.0000152587890625f));
-      }
-    }
+    for (int j = 0; j < 8; j++) V[hh * 8 + j] = fold_level2(p[j], __uint_as_float(a[j]));
+    tmem_ld8_wait(b);
+    tmem_ld8_start(t + 4 * TN, a);
 #pragma unroll
-    for (int j = 0; j < 16; j++) W[hh * 16 + j] = V[j] * 65536 + round_f2ll(cf[j] * 256.f);  // 256 c can pass 2^31
+    for (int j = 0; j < 8; j++) V[hh * 8 + j] += exact_f2i(__uint_as_float(b[j]));
+    tmem_ld8_wait(a);
+    tmem_ld8_start(t + 5 * TN, b);
+#pragma unroll
+    for (int j = 0; j < 8; j++) cf[hh * 8 + j] = __uint_as_float(a[j]);
+    tmem_ld8_wait(b);
+    tmem_ld8_start(t + 6 * TN, a);
+#pragma unroll
+    for (int j = 0; j < 8; j++) cf[hh * 8 + j] += __uint_as_float(b[j]) * 0.00390625f;
+    tmem_ld8_wait(a);
+#pragma unroll
+    for (int j = 0; j < 8; j++) cf[hh * 8 + j] += __uint_as_float(a[j]) * 0.0000152587890625f;
   }
+}
+
+// W = V 2^16 + round(256 c) of every column, in V's place (256 c can pass 2^31).
+__device__ __forceinline__ void emu_combine(long long (&V)[kEpiCols], const float (&cf)[kEpiCols]) {
+#pragma unroll
+  for (int j = 0; j < kEpiCols; j++) V[j] = V[j] * 65536 + round_f2ll(cf[j] * 256.f);
+  asm volatile("" ::: "memory");  // the loads of S stay behind: their registers are cf's
 }
 
 // S[row, col] += -W 2^{e_i + f_j - 56} for the thread's columns col = base +
 // cj, cj = cj0 .. cj0 + kEpiCols - 1, that lie below mcol and on or below the
-// diagonal; 16 loads of S in flight per thread.  Lane l's ebl is the exponent
+// diagonal; 8 loads of S in flight per thread.  Lane l's ebl is the exponent
 // f_j of column cj0 + l; every lane of the warp takes part (the exponents go
 // through shuffles).
 __device__ __forceinline__ void emu_apply(double* __restrict__ S, int n, int row, bool live_row, int base, int cj0,
                                           int mcol, int ea, int ebl, const long long (&W)[kEpiCols]) {
 #pragma unroll
-  for (int hh = 0; hh < kEpiCols / 16; hh++) {
-    double cur[16];
+  for (int hh = 0; hh < kEpiCols / 8; hh++) {
+    double cur[8];
 #pragma unroll
-    for (int j = 0; j < 16; j++) {
-      const int cj = cj0 + hh * 16 + j, col = base + cj;
+    for (int j = 0; j < 8; j++) {
+      const int cj = cj0 + hh * 8 + j, col = base + cj;
       cur[j] = (live_row && cj < mcol && row >= col) ? S[(int64_t)row + (int64_t)col * n] : 0.0;
     }
 #pragma unroll
-    for (int j = 0; j < 16; j++) {
-      const int c = hh * 16 + j, cj = cj0 + c, col = base + cj;
+    for (int j = 0; j < 8; j++) {
+      const int c = hh * 8 + j, cj = cj0 + c, col = base + cj;
       const int eb = __shfl_sync(0xffffffffu, ebl, c);
       const double nd = neg_scaled(W[c], ea + eb);
       if (live_row && cj < mcol && row >= col) S[(int64_t)row + (int64_t)col * n] = cur[j] + nd;
@@ -731,10 +757,12 @@ __global__ void __launch_bounds__(kEmuThreads, 1)
       }
       asm volatile("tcgen05.fence::after_thread_sync;");
       long long W[kEpiCols];
-      emu_fold(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)cbase, W);
+      float cf[kEpiCols];
+      emu_drain(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)cbase, W, cf);
       asm volatile("tcgen05.fence::before_thread_sync;");
       __syncwarp();
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_tempty)) : "memory");
+      emu_combine(W, cf);
       emu_apply(S, n, row, live_row, base, cj0, mcol, ea, ebl[0], W);
     }
   }
@@ -982,7 +1010,9 @@ __global__ void __launch_bounds__(256, 1) k_tc_panel_emu(double* __restrict__ S0
     const int ea = pow2_exponent(live_row ? scaleA[rho] : 1.0) - 56;
     const int ebl = pow2_exponent(cbase + lane < kb ? scaleB[cbase + lane] : 1.0);
     long long W[kEpiCols];
-    emu_fold(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)cbase, W);
+    float cf[kEpiCols];
+    emu_drain(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)cbase, W, cf);
+    emu_combine(W, cf);
 #pragma unroll
     for (int c = 0; c < kEpiCols; c++) {
       const int j = cbase + c;
@@ -1299,10 +1329,12 @@ __global__ void __launch_bounds__(kEmuThreads, 1)
       }
       asm volatile("tcgen05.fence::after_thread_sync;");
       long long W[kEpiCols];
-      emu_fold(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)cbase, W);
+      float cf[kEpiCols];
+      emu_drain(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)cbase, W, cf);
       asm volatile("tcgen05.fence::before_thread_sync;");
       __syncwarp();
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_tempty)) : "memory");
+      emu_combine(W, cf);
       emu_apply(S, n, row, live_row, base, cj0, m, ea, ebl[0], W);
     }
   }

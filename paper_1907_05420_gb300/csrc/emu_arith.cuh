@@ -151,6 +151,14 @@ KKT_HD int exact_f2i(float x) {
   return (bits_of(r) - kMagicBits) * 256 + (bits_of(lo + kMagic) - kMagicBits);
 }
 
+// x an integer-valued FP32 number, |x| <= 2^22: x as int32.
+KKT_HD int small_f2i(float x) { return bits_of(x + kMagic) - kMagicBits; }
+
+// The exact integer ((x0 256 + x1) 256 + x2) 256 + x3 of the digit-product levels
+// 0 to 3, |x0| <= 2^22, |x1| <= 2^23, |x2| and |x3| <= 2^24 (x0 256 + x1 fits 32 bits).
+KKT_HD int fold_level1(int p, float x1) { return p * 256 + exact_f2i(x1); }
+KKT_HD long long fold_level2(int p, float x2) { return (long long)p * 65536 + (long long)exact_f2i(x2) * 256; }
+
 // round-to-nearest-even of an FP32 x, |x| < 2^37, as int64
 // (x = 65536 hi + lo with hi = rn(x / 65536), lo exact, |lo| <= 2^15).
 KKT_HD long long round_f2ll(float x) {

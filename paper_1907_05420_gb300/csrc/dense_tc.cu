@@ -1048,27 +1048,34 @@ __global__ void __launch_bounds__(256, 1) k_tc_panel_emu(double* __restrict__ S0
 // only where their partial sums pass 2^24, which keeps the error of the
 // product within the worst-case rounding of an FP64 dot product of 256 terms.
 //
-// Image layout (per matrix and operand): 64-row blocks; in a block, for each
-// 32-column K chunk (8 of them) and each digit slice (7), the 8 row groups x 4
-// core matrices along K x 128 bytes (4 KB).  One shared-memory stage holds one
-// K chunk of a 128 x 64 tile: A 7 x 8 KB, B 7 x 4 KB.
+// Image layout (per matrix and operand): blocks of 128 rows (A) or 64 (B); in a
+// block, for each 16-column K chunk (16 of them) and each digit slice (7), the
+// row groups x 2 core matrices along K x 128 bytes (4 KB for A, 2 KB for B), so
+// that a block's chunk is one contiguous piece with all its slices.  One
+// shared-memory stage holds one K chunk of a 128 x 64 tile, A 28 KB and B 14 KB.
+// Five stages keep 170 KB of copies in flight under the products; two stages of
+// 32 columns, where a stage had to arrive during the other one's 1,800 cycles of
+// products, left the tensor pipe waiting for them.  9,241 buses: 107.7 -> 101.6
+// ms.
 constexpr int kEwW = 256;                          // outer panel width
-constexpr int kEwChunk = 32;                       // K per stage
-constexpr int kEwChunks = kEwW / kEwChunk;         // 8
-constexpr int kEwPiece = 4096;                     // one (block, chunk, slice): 8 row groups x 4 x 128 B
-constexpr int kEwBlockBytes = kEwChunks * kEmuSlices * kEwPiece;  // 64 rows: 229,376 bytes
-constexpr int kEwStageA = kEmuSlices * 2 * kEwPiece;  // 128 rows, 57,344 bytes
-constexpr int kEwStageB = kEmuSlices * kEwPiece;      // 64 rows, 28,672 bytes
-constexpr int kEwStages = 2;
-__host__ __device__ constexpr int ew_smem_bytes() { return kEwStages * (kEwStageA + kEwStageB); }  // 168 KB
+constexpr int kEwChunk = 16;                       // K per stage
+constexpr int kEwChunks = kEwW / kEwChunk;         // 16
+constexpr int kEwPieceA = 4096, kEwPieceB = 2048;  // one (block, chunk, slice)
+constexpr int kEwBlockBytes = kEwChunks * kEmuSlices * kEwPieceB;  // 64 rows: 229,376 bytes
+constexpr int kEwStageA = kEmuSlices * kEwPieceA;  // 128 rows, 28,672 bytes
+constexpr int kEwStageB = kEmuSlices * kEwPieceB;  // 64 rows, 14,336 bytes
+constexpr int kEwStages = 5;
+constexpr int kEwWarpCols = kEwW / 8;              // columns a warp of the slicing kernels takes
+__host__ __device__ constexpr int ew_smem_bytes() { return kEwStages * (kEwStageA + kEwStageB); }  // 210 KB
 
-// The digit images of a thread's 32 columns (K chunk k) of row rho of an operand.
-__device__ __forceinline__ void slice_chunk(const double (&v)[kEwChunk], int e_exp, uint8_t* img, int rho, int k,
-                                            const uint32_t* table) {
-  const int blk = rho >> 6, rr = rho & 63, g = rr >> 3, r8 = rr & 7;
-  uint8_t* bimg = img + (int64_t)blk * kEwBlockBytes + (g * 4) * 128 + r8 * 16;
+// The digit images of a thread's 32 columns (32 warp ..) of row rho of operand A
+// or B.
+__device__ __forceinline__ void slice_columns(const double (&v)[kEwWarpCols], int e_exp, uint8_t* img, int rho, bool isA,
+                                              int warp, const uint32_t* table) {
+  const int rows_blk = isA ? TM : TN, piece = isA ? kEwPieceA : kEwPieceB, rr = rho & (rows_blk - 1);
+  uint8_t* bimg = img + (int64_t)(rho / rows_blk) * kEwChunks * kEmuSlices * piece + (rr >> 3) * 256 + (rr & 7) * 16;
 #pragma unroll
-  for (int kq = 0; kq < 4; kq++) {
+  for (int kq = 0; kq < kEwWarpCols / 8; kq++) {
     uint32_t packed[kEmuSlices][4];
 #pragma unroll
     for (int e = 0; e < 8; e++) {
@@ -1084,9 +1091,10 @@ __device__ __forceinline__ void slice_chunk(const double (&v)[kEwChunk], int e_e
         packed[sl][e >> 1] = (e & 1) ? (packed[sl][e >> 1] | (hbits << 16)) : hbits;
       }
     }
+    uint8_t* dst = bimg + (int64_t)((warp * 2 + (kq >> 1)) * kEmuSlices) * piece + (kq & 1) * 128;
 #pragma unroll
     for (int sl = 0; sl < kEmuSlices; sl++)
-      *reinterpret_cast<uint4*>(bimg + ((int64_t)(k * kEmuSlices + sl)) * kEwPiece + kq * 128) =
+      *reinterpret_cast<uint4*>(dst + sl * piece) =
           make_uint4(packed[sl][0], packed[sl][1], packed[sl][2], packed[sl][3]);
   }
 }
@@ -1094,8 +1102,7 @@ __device__ __forceinline__ void slice_chunk(const double (&v)[kEwChunk], int e_e
 // rows rho in [0, mpad) of the outer trailing matrix of matrix blockIdx.y:
 // operand A = rows of Y (columns 0..kw-1 of Yw, leading dimension n), operand
 // B = rows of L (columns K0..K0+kw-1 of S); rows >= m and columns >= kw are zero.
-// 32 rows of one operand per CTA: lane l takes row l, warp w the K chunk w (32
-// columns), read once, all loads in flight together, and kept in registers
+// 32 rows of one operand per CTA: lane l takes row l, warp w the columns 32 w .., read once, all loads in flight together, and kept in registers
 // while the row's scale is found.  One matrix of order 1,848: 8.4 us (106 with a
 // thread per row that read its 256 columns twice), 24 of order 7,000: 108 us
 // (281).
@@ -1105,30 +1112,29 @@ __global__ void __launch_bounds__(256, 2) k_slice_wide(const double* __restrict_
                                                     double* __restrict__ scaleA0, double* __restrict__ scaleB0,
                                                     int64_t s_stride, int64_t y_stride, int64_t img_stride,
                                                     int64_t scale_stride) {
-  static_assert(kEwChunks == 8, "a warp per K chunk");
   __shared__ unsigned long long mx[8][32];
   __shared__ uint32_t bf16_of_byte[256];
   const int64_t bb = blockIdx.y;
   bf16_of_byte[threadIdx.x] = bf16_bits_of_byte(threadIdx.x);
-  const int k = threadIdx.x >> 5;  // K chunk
+  const int k = threadIdx.x >> 5;  // columns 32 k ..
   const int q = blockIdx.x * 32 + (threadIdx.x & 31);
   const bool isA = q < mpad;
   const int rho = isA ? q : q - mpad;
   const bool live = rho < m;
   const double* src = (isA ? Yw0 + bb * y_stride : S0 + bb * s_stride + (int64_t)K0 * n) + (base + rho);
-  double v[kEwChunk];
+  double v[kEwWarpCols];
   unsigned long long mag = 0;
 #pragma unroll
-  for (int e = 0; e < kEwChunk; e++) {
-    const int c = k * kEwChunk + e;
+  for (int e = 0; e < kEwWarpCols; e++) {
+    const int c = k * kEwWarpCols + e;
     v[e] = live && c < kw ? src[(int64_t)c * n] : 0.0;
   }
 #pragma unroll
-  for (int e = 0; e < kEwChunk; e++) mag = max(mag, magnitude_bits(v[e]));
+  for (int e = 0; e < kEwWarpCols; e++) mag = max(mag, magnitude_bits(v[e]));
   mag = max_over_warps(mag, mx);  // (its barrier covers the table too)
   const int e_exp = mag ? scale_exponent(mag) + 1 : 0;  // |v| < 2^(e-1)
   if (k == 0) (isA ? scaleA0 : scaleB0)[bb * scale_stride + rho] = ldexp(1.0, e_exp);
-  slice_chunk(v, e_exp, (isA ? imgA0 : imgB0) + bb * img_stride, rho, k, bf16_of_byte);
+  slice_columns(v, e_exp, (isA ? imgA0 : imgB0) + bb * img_stride, rho, isA, k, bf16_of_byte);
 }
 
 // The operands of the tail's heavy update (matrix blockIdx.y), straight from the
@@ -1150,17 +1156,17 @@ __global__ void __launch_bounds__(256, 2) k_slice_heavy(const double* __restrict
   __shared__ uint32_t bf16_of_byte[256];
   const int64_t bb = blockIdx.y;
   bf16_of_byte[threadIdx.x] = bf16_bits_of_byte(threadIdx.x);
-  const int k = threadIdx.x >> 5;  // K chunk
+  const int k = threadIdx.x >> 5;  // columns 32 k ..
   const int q = blockIdx.x * 32 + (threadIdx.x & 31);
   const bool isA = q < mpad;
   const int rho = isA ? q : q - mpad;
   const double* L = Lx + bb * pt;
   const double* P = isA ? LDx + bb * ldt : L;
-  double v[kEwChunk];
+  double v[kEwWarpCols];
   unsigned long long mag = 0;
 #pragma unroll
-  for (int e = 0; e < kEwChunk; e++) {
-    const int c = k * kEwChunk + e;
+  for (int e = 0; e < kEwWarpCols; e++) {
+    const int c = k * kEwWarpCols + e;
     v[e] = 0.0;
     if (c < ncol && rho < nT) {
       const int i = pos[(int64_t)sn[c] * nT + rho];
@@ -1171,21 +1177,21 @@ __global__ void __launch_bounds__(256, 2) k_slice_heavy(const double* __restrict
     }
   }
 #pragma unroll
-  for (int e = 0; e < kEwChunk; e++) mag = max(mag, magnitude_bits(v[e]));
+  for (int e = 0; e < kEwWarpCols; e++) mag = max(mag, magnitude_bits(v[e]));
   mag = max_over_warps(mag, mx);  // (its barrier covers the table too)
   const int e_exp = mag ? scale_exponent(mag) + 1 : 0;  // |v| < 2^(e-1)
   if (k == 0) (isA ? scaleA0 : scaleB0)[bb * scale_stride + rho] = ldexp(1.0, e_exp);
-  slice_chunk(v, e_exp, (isA ? imgA0 : imgB0) + bb * img_stride, rho, k, bf16_of_byte);
+  slice_columns(v, e_exp, (isA ? imgA0 : imgB0) + bb * img_stride, rho, isA, k, bf16_of_byte);
 }
 
 // The K = 256 emulated update: one CTA per run of up to kEmuRun tiles (I, J)
 // of one tile row I (128 x 64 tiles of the lower triangle, J <= 2I + 1);
 // jmode 1 takes J < 4 (the next outer panel's 256 columns), 2 the rest.
 // Warp roles as in k_tc_update_emu: warp 0 copies the K chunks of A and B of
-// every tile through two shared-memory stages, warp 1 issues the 56 MMAs of
-// each chunk (28 digit pairs x 2 K steps of 16) into 7 tensor-memory levels,
-// warps 2..9 fold the levels of a finished tile, hand tensor memory back and
-// read-modify-write S.  Every wait is bounded, as there.
+// every tile through the shared-memory stages, warp 1 issues the MMAs of each
+// chunk (mma_digit_pairs) into 7 tensor-memory levels, warps 2..9 drain the
+// levels of a finished tile, hand tensor memory back and read-modify-write S.
+// Every wait is bounded, as there.
 __global__ void __launch_bounds__(kEmuThreads, 1)
     k_tc_update_emu_wide(double* __restrict__ S0, int n, int base, int m, int TI, int TJ, int jmode, int nchunk,
                          const uint8_t* __restrict__ imgA0, const uint8_t* __restrict__ imgB0,
@@ -1230,11 +1236,11 @@ __global__ void __launch_bounds__(kEmuThreads, 1)
 
   if (warp == 0) {
     if (lane == 0 && ntile > 0) {
-      // producer: chunk g = u * nchunk + k of tile u into stage g & 1
-      int armed[kEwStages] = {0, 0};
-      for (int g = 0; g < nsteps; g++) {
-        const int st = g & 1, u = g / nchunk, k = g - u * nchunk, J = j0 + u;
-        if (g >= kEwStages && !mbar_wait_ab(smem_u32(&bar_empty[st]), (uint32_t)(((g >> 1) - 1) & 1), &s_abort)) {
+      // producer: chunk g = u * nchunk + k of tile u into stage g mod kEwStages
+      int g = 0, st = 0, u = 0, k = 0;
+      uint32_t par = 1;  // parity of the stage's last release, once it has been used
+      for (; g < nsteps; g++) {
+        if (g >= kEwStages && !mbar_wait_ab(smem_u32(&bar_empty[st]), par, &s_abort)) {
           if (!s_abort) atomicExch(err, 13);
           s_abort = 1;
           break;
@@ -1244,24 +1250,29 @@ __global__ void __launch_bounds__(kEmuThreads, 1)
                      "r"((uint32_t)(kEwStageA + kEwStageB))
                      : "memory");
         uint8_t* sA = smem + st * (kEwStageA + kEwStageB);
-        uint8_t* sB = sA + kEwStageA;
-        for (int sl = 0; sl < kEmuSlices; sl++) {
-          const int64_t piece = ((int64_t)k * kEmuSlices + sl) * kEwPiece;
-          bulk_load(sA + sl * 2 * kEwPiece, imgA + (int64_t)(2 * I) * kEwBlockBytes + piece, kEwPiece, bf);
-          bulk_load(sA + sl * 2 * kEwPiece + kEwPiece, imgA + (int64_t)(2 * I + 1) * kEwBlockBytes + piece, kEwPiece,
-                    bf);
-          bulk_load(sB + sl * kEwPiece, imgB + (int64_t)J * kEwBlockBytes + piece, kEwPiece, bf);
+        bulk_load(sA, imgA + (int64_t)(2 * I) * kEwBlockBytes + (int64_t)k * kEwStageA, kEwStageA, bf);
+        bulk_load(sA + kEwStageA, imgB + (int64_t)(j0 + u) * kEwBlockBytes + (int64_t)k * kEwStageB, kEwStageB, bf);
+        if (++k == nchunk) {
+          k = 0;
+          u++;
         }
-        armed[st]++;
+        if (++st == kEwStages) {
+          st = 0;
+          par ^= 1;
+        }
       }
+      // the copies issued must land before the CTA's shared memory goes away
       volatile int never = 0;
-      for (int st = 0; st < kEwStages; st++)
-        if (armed[st] > 0) mbar_wait_ab(smem_u32(&bar_full[st]), (uint32_t)((armed[st] - 1) & 1), &never);
+      for (int q = 0; q < kEwStages; q++) {
+        const int loads = (g - q + kEwStages - 1) / kEwStages;  // into stage q
+        if (loads > 0) mbar_wait_ab(smem_u32(&bar_full[q]), (uint32_t)((loads - 1) & 1), &never);
+      }
     }
   } else if (warp == 1) {
     if (lane == 0 && ntile > 0) {
       // MMA issuer
-      uint32_t last_bar = 0, last_par = 0;
+      uint32_t last_bar = 0, last_par = 0, par = 0;
+      int st = 0;
       bool stop = false;
       for (int u = 0; u < ntile && !stop; u++) {
         if (u >= 1 && !mbar_wait_ab(smem_u32(&bar_tempty), (uint32_t)((u - 1) & 1), &s_abort)) {
@@ -1271,8 +1282,7 @@ __global__ void __launch_bounds__(kEmuThreads, 1)
         }
         asm volatile("tcgen05.fence::after_thread_sync;");
         for (int k = 0; k < nchunk; k++) {
-          const int g = u * nchunk + k, st = g & 1;
-          if (!mbar_wait_ab(smem_u32(&bar_full[st]), (uint32_t)((g >> 1) & 1), &s_abort)) {
+          if (!mbar_wait_ab(smem_u32(&bar_full[st]), par, &s_abort)) {
             if (!s_abort) atomicExch(err, 15);
             s_abort = 1;
             stop = true;
@@ -1280,17 +1290,16 @@ __global__ void __launch_bounds__(kEmuThreads, 1)
           }
           asm volatile("tcgen05.fence::after_thread_sync;");
           const uint8_t* sA = smem + st * (kEwStageA + kEwStageB);
-          const uint64_t a0 = umma_desc(smem_u32(sA), 128, 512);
-          const uint64_t b0 = umma_desc(smem_u32(sA + kEwStageA), 128, 512);
-#pragma unroll
-          for (int ks = 0; ks < kEwChunk / 16; ks++)
-            mma_digit_pairs(tmem, umma_desc_at(a0, ks * 256), 2 * kEwPiece, umma_desc_at(b0, ks * 256), kEwPiece,
-                            k == 0 && ks == 0);
-          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                           smem_u32(&bar_empty[st]))
-                       : "memory");
+          mma_digit_pairs(tmem, umma_desc(smem_u32(sA), 128, 256), kEwPieceA,
+                          umma_desc(smem_u32(sA + kEwStageA), 128, 256), kEwPieceB, k == 0);
           last_bar = smem_u32(&bar_empty[st]);
-          last_par = (uint32_t)((g >> 1) & 1);
+          last_par = par;
+          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(last_bar)
+                       : "memory");
+          if (++st == kEwStages) {
+            st = 0;
+            par ^= 1;
+          }
         }
         if (stop) break;
         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(

@@ -85,6 +85,9 @@ void free_all(Handle* h) {
   if (h->factor_exec) cudaGraphExecDestroy(h->factor_exec);
   for (cudaGraphExec_t ex : h->solve_exec)
     if (ex) cudaGraphExecDestroy(ex);
+  for (auto& kind : h->app_exec)
+    for (cudaGraphExec_t ex : kind)
+      if (ex) cudaGraphExecDestroy(ex);
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
   if (h->side_stream) cudaStreamDestroy(h->side_stream);
   if (h->early_stream) cudaStreamDestroy(h->early_stream);
@@ -1070,6 +1073,52 @@ void build_solve_graph(Handle& h) {
   }
 }
 
+// kkt_solve's host loop up to its next look at the norms: the application of
+// the factorization to h.rhs into h.x, or with `refine` to the residual and x +=
+// dx; then the residual, its norms and what the test reads.
+cudaError_t enqueue_apply(Handle& h, bool refine, cudaStream_t st) {
+  cudaError_t e = refine ? launch_apply_inverse(h, h.rho, h.dx, st) : launch_apply_inverse(h, h.rhs, h.x, st);
+  if (e == cudaSuccess && refine) e = launch_axpy(h, h.x, h.dx, (int64_t)h.N * h.nA + h.nC, st);
+  if (e == cudaSuccess) e = launch_residual(h, h.rhs, h.x, h.rho, st);
+  if (e == cudaSuccess) e = launch_norms(h, h.rho, h.x, h.rhs, st);
+  return e == cudaSuccess ? launch_publish(h, st) : e;
+}
+
+// The same as a CUDA graph from the handle's second such call on (use_graphs;
+// the arguments are the handle's buffers): some 30 dependent launches of a few
+// microseconds, which the host issues more slowly than a small system runs them
+// (30 buses x 24 periods: a solve 195 us directly, 137 us so; factor and solve
+// 530 and 465 us).
+// A handle that solves once does not pay for the capture.
+cudaError_t run_apply(Handle& h, bool refine, cudaStream_t st) {
+  const int sf = h.s_factor, kind = refine ? 1 : 0;
+  if (!h.opt.use_graphs || h.app_seen[sf][kind] < 0 || h.app_seen[sf][kind]++ == 0) return enqueue_apply(h, refine, st);
+  cudaGraphExec_t& exec = h.app_exec[sf][kind];
+  if (!exec) {
+    const int64_t l0 = h.launches;
+    cudaGraph_t g = nullptr;
+    cudaError_t e = cudaStreamBeginCapture(h.cap_stream, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+      const cudaError_t e1 = enqueue_apply(h, refine, h.cap_stream);
+      const cudaError_t e2 = cudaStreamEndCapture(h.cap_stream, &g);
+      e = e1 != cudaSuccess ? e1 : e2;
+    }
+    if (e == cudaSuccess && g) e = cudaGraphInstantiate(&exec, g, 0);
+    if (g) cudaGraphDestroy(g);
+    h.app_launches[sf][kind] = h.launches - l0;
+    h.launches = l0;
+    if (e != cudaSuccess || !exec) {
+      exec = nullptr;
+      h.app_seen[sf][kind] = -1;  // launch directly from now on
+      (void)cudaGetLastError();
+      return enqueue_apply(h, refine, st);
+    }
+  }
+  h.app_seen[sf][kind] = 1;
+  h.launches += h.app_launches[sf][kind];
+  return cudaGraphLaunch(exec, st);
+}
+
 // One cycle of GMRES refinement (right preconditioning by the factorization
 // K~): from the residual rho = r - K x in h->rho, up to `budget` Krylov steps
 // z_j = K~^{-1} v_j, w = K z_j, modified Gram-Schmidt against v_0..v_j, Givens
@@ -1356,6 +1405,7 @@ kkt_status kkt_solve(kkt_handle* hh, const double* rhs, double* x, int32_t nrhs,
     const bool on_graph = h->opt.device_refine && !early && h->solve_exec[sf];
     int steps = 0, before_fallback = 0;  // steps of this refinement, of the one before the FP64 fallback
     bool nonfinite = false, host_loop = true;
+    bool published = false;  // the norms of the current iterate are on their way to the host
     double eta = INFINITY, eta_prev = INFINITY;
     if (on_graph) {
       // the application and the refinement loop on the device; one read of the outcome
@@ -1405,16 +1455,17 @@ kkt_status kkt_solve(kkt_handle* hh, const double* rhs, double* x, int32_t nrhs,
     } else {
       KKT_CUDA(cudaMemcpyAsync(h->rhs, rq, sizeof(double) * nK,
                                on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st));
-      KKT_CUDA(launch_apply_inverse(*h, h->rhs, h->x, st));
+      KKT_CUDA(run_apply(*h, false, st));
+      published = true;
     }
     h->schur_pending = false;
     while (host_loop) {
-      KKT_CUDA(launch_residual(*h, h->rhs, h->x, h->rho, st));
-      KKT_CUDA(launch_norms(*h, h->rho, h->x, h->rhs, st));
-      KKT_CUDA(cudaMemcpyAsync(h->host_red, h->red, sizeof(double) * 3, cudaMemcpyDeviceToHost, st));
-      KKT_CUDA(cudaMemcpyAsync(h->host_red + 3, h->knorm, sizeof(double), cudaMemcpyDeviceToHost, st));
-      KKT_CUDA(cudaMemcpyAsync(h->host_red + 4, h->dev_err, sizeof(int), cudaMemcpyDeviceToHost, st));
-      if (h->cum) KKT_CUDA(cudaMemcpyAsync(h->host_red + 5, h->cum_err, sizeof(int), cudaMemcpyDeviceToHost, st));
+      if (!published) {
+        KKT_CUDA(launch_residual(*h, h->rhs, h->x, h->rho, st));
+        KKT_CUDA(launch_norms(*h, h->rho, h->x, h->rhs, st));
+        KKT_CUDA(launch_publish(*h, st));
+      }
+      published = false;
       KKT_CUDA(cudaStreamSynchronize(st));
       if (*reinterpret_cast<int*>(h->host_red + 4) != 0) {
         set_error("kkt_solve: a bounded device wait ran out");
@@ -1466,8 +1517,8 @@ kkt_status kkt_solve(kkt_handle* hh, const double* rhs, double* x, int32_t nrhs,
         steps += its;
         continue;
       }
-      KKT_CUDA(launch_apply_inverse(*h, h->rho, h->dx, st));
-      KKT_CUDA(launch_axpy(*h, h->x, h->dx, nK, st));
+      KKT_CUDA(run_apply(*h, true, st));
+      published = true;
       steps++;
     }
     KKT_CUDA(cudaMemcpyAsync(xq, h->x, sizeof(double) * nK,

@@ -258,6 +258,11 @@ struct Handle {
   cudaGraphExec_t solve_exec[2] = {nullptr, nullptr};
   bool solve_graph_failed[2] = {false, false};
   double* rstate = nullptr;
+  // graphs of kkt_solve's host loop, per kind of factor of S: [0] the first
+  // application with its residual and norms, [1] one refinement step with them
+  cudaGraphExec_t app_exec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
+  int64_t app_launches[2][2] = {{0, 0}, {0, 0}};
+  int app_seen[2][2] = {{0, 0}, {0, 0}};
   // structured S of the cumulative coupling (structured_s = 2, cumulative.cu):
   // ns x ns blocks, column-major, N of each unless noted
   bool cum = false;
@@ -387,6 +392,8 @@ cudaError_t launch_knorm(Handle& h, cudaStream_t st);
 cudaError_t launch_axpy(Handle& h, double* y, const double* x, int64_t n, cudaStream_t st);
 cudaError_t launch_norms(Handle& h, const double* rho, const double* x, const double* rhs,
                          cudaStream_t st);
+// the norms (h.red), ||K||_inf, dev_err and cum_err to host_red[0..5]
+cudaError_t launch_publish(Handle& h, cudaStream_t st);
 // GMRES refinement: deterministic dot product into device *out (scratch red[16..16+512)), y += a x, y = a x
 cudaError_t launch_dot(Handle& h, const double* a, const double* b, int64_t n, double* out, cudaStream_t st);
 cudaError_t launch_axpby(Handle& h, double* y, double a, const double* x, int64_t n, cudaStream_t st);

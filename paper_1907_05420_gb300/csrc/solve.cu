@@ -512,6 +512,17 @@ __device__ __forceinline__ void block_max_to(double* out, double m) {
   }
 }
 
+// What kkt_solve's convergence test reads, straight into pinned host memory (one
+// launch instead of a copy for each).
+__global__ void k_publish(const double* __restrict__ red, const double* __restrict__ knorm,
+                          const int* __restrict__ dev_err, const int* __restrict__ cum_err, double* host) {
+  const int l = threadIdx.x;
+  if (l < 3) host[l] = red[l];
+  if (l == 3) host[3] = knorm[0];
+  if (l == 4) *reinterpret_cast<int*>(host + 4) = *dev_err;
+  if (l == 5) *reinterpret_cast<int*>(host + 5) = cum_err ? *cum_err : 0;
+}
+
 // ||K||_inf: row sums of |K| (NaN if an entry of A or B is NaN)
 __global__ void k_knorm_blocks(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ src,
                                const double* __restrict__ a_vals, int64_t nnzA,
@@ -811,6 +822,12 @@ cudaError_t launch_norms(Handle& h, const double* rho, const double* x, const do
     k_norms3<<<grid_for(nK), 256, 0, st>>>(rho, x, rhs, nK, h.red);
     h.launches++;
   }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_publish(Handle& h, cudaStream_t st) {
+  k_publish<<<1, 32, 0, st>>>(h.red, h.knorm, h.dev_err, h.cum ? h.cum_err : nullptr, h.host_red);
+  h.launches++;
   return cudaGetLastError();
 }
 

@@ -63,7 +63,7 @@ void free_all(Handle* h) {
                   h->d.b_blockptr, h->d.e_t, h->d.e_block, h->d.wpos, h->d.sn_wrow, h->d.w_dpos,
                   h->d.w_col, h->d.reach_lvl_sn, h->d.s_key, h->d.s_ptr, h->d.s_e1, h->d.s_e2,
                   h->d.t_ptr, h->d.t_e, h->d.bt_ptr, h->d.E, h->d.g_rows, h->d.trsv_jlo, h->d.trsv_jhi,
-                  h->d.flvl_sn, h->d.flvl_desc, h->d.fr_ptr, h->d.fr_rec, h->d.wr_ptr, h->d.wr_row, h->d.w_sn, h->d.twork, h->d.tpairs, h->d.upd_ntail, h->d.reach_lvl_sn_nt, h->d.tail_sn_list, h->d.hv_off, h->d.hv_sn, h->d.hv_col, h->d.hv_pos, h->d.tail_wrow, h->d.wt_ptr, h->d.wt_idx,
+                  h->d.panel_small, h->d.panel_items, h->d.flvl_desc, h->d.fr_ptr, h->d.fr_rec, h->d.wr_ptr, h->d.wr_row, h->d.w_sn, h->d.twork, h->d.tpairs, h->d.upd_ntail, h->d.reach_lvl_sn_nt, h->d.tail_sn_list, h->d.hv_off, h->d.hv_sn, h->d.hv_col, h->d.hv_pos, h->d.tail_wrow, h->d.wt_ptr, h->d.wt_idx,
                   h->d.g_key, h->d.g_ptr, h->d.g_row, h->Xinv, h->Sdinv, h->wdinv, h->Xtail, h->Tt, h->TY, h->t_imgA, h->t_imgB,
                   h->t_scaleA, h->t_scaleB, h->Lx, h->LDx, h->a_vals, h->b_vals,
                   h->c_vals, h->anorm, h->W, h->G, h->S, h->Ypanel, h->knorm, h->counters, h->r,
@@ -577,6 +577,31 @@ kkt_status analyze_one(const kkt_pattern* pat, const kkt_options* opt, double ta
       fr_rec.resize(fr_ptr[n]);
     }
   }
+  std::vector<SnDesc> panel_small;
+  std::vector<PanelItem> panel_items;
+  h->panel_lvl.assign(S.nlevels, PanelLevel{});
+  for (int l = 0; l < S.nlevels; l++) {
+    PanelLevel& L = h->panel_lvl[l];
+    std::vector<PanelItem> second;
+    L.small0 = (int32_t)panel_small.size();
+    L.item0 = (int32_t)panel_items.size();
+    for (int q = h->flvl_ptr[l]; q < h->flvl_ptr[l + 1]; q++) {
+      const int s = flvl_sn[q], f = S.sn_first[s], w = S.sn_first[s + 1] - f;
+      const int m = (int)(S.sn_rowptr[s + 1] - S.sn_rowptr[s]);
+      if (w * (int64_t)m <= kPanelSmall) {
+        panel_small.push_back(SnDesc{S.sn_valoff[s], S.sn_rowptr[s], f, w, m, 0});
+        continue;
+      }
+      const bool split = m - w > kPanelRows;
+      panel_items.push_back(PanelItem{S.sn_valoff[s], f, w, m, w, split ? w : m, 1});
+      for (int r = w; split && r < m; r += kPanelTile)
+        second.push_back(PanelItem{S.sn_valoff[s], f, w, m, r, std::min(m, r + kPanelTile), 0});
+    }
+    L.nsmall = (int32_t)panel_small.size() - L.small0;
+    L.nitems = (int32_t)panel_items.size() - L.item0;
+    L.nrows = (int32_t)second.size();
+    panel_items.insert(panel_items.end(), second.begin(), second.end());
+  }
   std::vector<SnDesc> flvl_desc;
   for (int s : flvl_sn)
     flvl_desc.push_back(SnDesc{S.sn_valoff[s], S.sn_rowptr[s], S.sn_first[s], S.sn_first[s + 1] - S.sn_first[s],
@@ -690,7 +715,8 @@ kkt_status analyze_one(const kkt_pattern* pat, const kkt_options* opt, double ta
   UP(diag_pos, diag_pos);
   UP(fwork, fwork);
   UP(fpairs, fpairs);
-  UP(flvl_sn, flvl_sn);
+  UP(panel_small, panel_small);
+  UP(panel_items, panel_items);
   UP(flvl_desc, flvl_desc);
   UP(fr_ptr, fr_ptr);
   UP(fr_rec, fr_rec);

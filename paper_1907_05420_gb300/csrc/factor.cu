@@ -13,7 +13,7 @@
 //     from its descendants d,  P_s[rel(i), j - f_s] -= sum_k L_d[i,k] D_d[k] L_d[j,k],
 //     one CTA per (32-row tile of s, block) so that the wide supernodes at the
 //     top of the tree spread over many SMs;
-//   k_panel_factor: dense LDL^T of the panel (1x1 pivots; a pivot below
+//   k_panel_factor: dense LDL^T of the panels (1x1 pivots; a pivot below
 //     pivot_eps*max|A_i| is replaced by the expected-sign value and counted).
 // The top of the tree (the dense tail, a suffix of the supernodes) is left out
 // of the level loop: once the rest is factored, its updates from outside the
@@ -140,53 +140,206 @@ __global__ void __launch_bounds__(kFactorThreads) k_factor_update(const int32_t*
   }
 }
 
-__global__ void __launch_bounds__(256) k_panel_factor(const int32_t* __restrict__ lvl_sn, DevSym d,
-                                                      double* __restrict__ Lx, int64_t pt,
-                                                      double* __restrict__ LDx, int64_t ldt,
-                                                      const double* __restrict__ anorm,
-                                                      double pivot_eps,
-                                                      unsigned long long* __restrict__ counters) {
-  const int s = lvl_sn[blockIdx.x], b = blockIdx.y;
-  const int m = (int)(d.sn_rowptr[s + 1] - d.sn_rowptr[s]);
-  const int f = d.sn_first[s], w = d.sn_first[s + 1] - f;
-  double* P = Lx + b * pt + d.sn_valoff[s];
-  const double thr = pivot_eps * anorm[b];
-  __shared__ double dsh, dinv_sh;
+// Dense LDL^T of the panels of one level (1x1 pivots; right-looking order of the
+// operations on every entry), and L D of each panel for the updates of its
+// ancestors: column c's entries times d_c, the product the updates would
+// otherwise form per target tile.  The leaves are thousands of panels of a few
+// columns and rows, the top of the tree a few of up to 32 columns and thousands
+// of rows, so a launch has two kinds of CTAs:
+//   small panels (at most kPanelSmall entries): eight lanes each, staged in shared
+//     memory, the blocks of one supernode side by side;
+//   items of a larger panel: its w x w triangle in shared memory, then one row per
+//     thread in registers against it.  A panel of more than kPanelRows rows below
+//     its triangle has an item for the triangle and, in a second launch, one per
+//     tile of kPanelTile rows.
+// Bound by the FP64 pipe and, at the top, by the chain of pivots.  With one CTA of
+// 256 threads per panel, working on it in global memory, all levels of 2,383 buses
+// x 96 periods took 1.55 ms, of 301 x 48 0.18 ms and of 9,241 x 24 10 ms (there
+// panels of 32 columns and thousands of rows); now 0.63, 0.093 and 1.39 ms.
+constexpr int kPanelThreads = 128;
+constexpr int kPanelGroups = kPanelThreads / 8;
+
+struct PanelSmallShared {
+  double t[kPanelGroups][kPanelSmall + 1];
+};
+struct PanelTileShared {
+  double T[kMaxSnWidth][kMaxSnWidth + 1];
+  double U[kMaxSnWidth][kMaxSnWidth];  // U[c][r] = l_rc d_c (0 from column w on)
+  double D[kMaxSnWidth], Di[kMaxSnWidth];  // d_c and 1 / d_c (0 from column w on)
+};
+
+// The pivot as it is used: a magnitude below thr becomes +-thr (thr > 0).  Bit
+// patterns of non-negative numbers order as the numbers do; a NaN stays.
+// cnt: positive, negative, zero or NaN, perturbed.
+__device__ __forceinline__ double panel_pivot(double dv, double thr, bool primal, int* cnt, bool count) {
+  const long long inf = 0x7ff0000000000000LL;
+  const long long mag = __double_as_longlong(dv) & 0x7fffffffffffffffLL;
+  const bool pert = mag < __double_as_longlong(thr);
+  if (pert) dv = primal ? thr : -thr;
+  if (count) {
+    const long long v = __double_as_longlong(dv), m = v & 0x7fffffffffffffffLL;
+    atomicAdd(&cnt[m == 0 || m > inf ? 2 : (v > 0 ? 0 : 1)], 1);
+    if (pert) atomicAdd(&cnt[3], 1);
+  }
+  return dv;
+}
+
+__device__ __forceinline__ void panel_small(PanelSmallShared& sh, const SnDesc* __restrict__ small, int nsmall, int cta,
+                                            const int32_t* __restrict__ col_primal, double* __restrict__ Lx,
+                                            int64_t pt, double* __restrict__ LDx, int64_t ldt,
+                                            const double* __restrict__ anorm, double pivot_eps, int N, int* cnt) {
+  const int g = threadIdx.x >> 3, l = threadIdx.x & 7;
+  const int64_t q = (int64_t)cta * kPanelGroups + g;
+  const bool on = q < (int64_t)nsmall * N;
+  const int b = on ? (int)(q % N) : 0;
+  SnDesc S{};
+  if (on) S = small[q / N];
+  const int w = on ? S.w : 0, m = S.m;
+  double* T = sh.t[g];
+  double* P = Lx + b * pt + S.val;
+  double* PD = LDx + b * ldt + S.val;
+  const double thr = on ? pivot_eps * anorm[b] : 0.0;
+  for (int e = l; e < w * m; e += 8) T[e] = P[e];
+  const int wmax = __reduce_max_sync(0xffffffffu, w);
+  __syncwarp();
+  for (int c = 0; c < wmax; c++) {
+    const bool act = c < w;
+    double* colc = T + c * m;
+    double dv = 0.0;
+    if (act) {
+      dv = panel_pivot(colc[c], thr, col_primal[S.f + c] != 0, cnt, l == 0);
+      const double di = pivot_recip(dv);
+      for (int r = c + 1 + l; r < m; r += 8) colc[r] *= di;
+    }
+    __syncwarp();
+    if (act) {
+      if (l == 0) colc[c] = dv;
+      for (int c2 = c + 1; c2 < w; c2++) {
+        const double l2 = colc[c2] * dv;
+        for (int r = c2 + l; r < m; r += 8) T[c2 * m + r] -= colc[r] * l2;
+      }
+    }
+    __syncwarp();
+  }
+  for (int c = 0; c < w; c++) {
+    const double dv = T[c * m + c];
+    for (int r = l; r < m; r += 8) {
+      const double v = T[c * m + r];
+      P[c * m + r] = v;
+      PD[c * m + r] = v * dv;
+    }
+  }
+}
+
+// one row per thread, eight columns of it in registers at a time (the sums read
+// earlier columns again from L1; their FP64 operations take far longer)
+__device__ __forceinline__ void panel_rows(const PanelTileShared& sh, double* P, double* PD, int m, int w, int r0,
+                                           int r1) {
+  constexpr int W = 8;
+  for (int r = r0 + threadIdx.x; r < r1; r += kPanelThreads) {
+    for (int c0 = 0; c0 < w; c0 += W) {
+      double a[W];
+#pragma unroll
+      for (int c = 0; c < W; c++) a[c] = c0 + c < w ? P[(int64_t)(c0 + c) * m + r] : 0.0;
+#pragma unroll 4
+      for (int k = 0; k < c0; k++) {
+        const double lk = P[(int64_t)k * m + r];
+#pragma unroll
+        for (int c = 0; c < W; c++) a[c] -= lk * sh.U[k][c0 + c];
+      }
+#pragma unroll
+      for (int c = 0; c < W; c++) {
+        a[c] *= sh.Di[c0 + c];
+#pragma unroll
+        for (int c2 = c + 1; c2 < W; c2++) a[c2] -= a[c] * sh.U[c0 + c][c0 + c2];
+      }
+#pragma unroll
+      for (int c = 0; c < W; c++)
+        if (c0 + c < w) {
+          P[(int64_t)(c0 + c) * m + r] = a[c];
+          PD[(int64_t)(c0 + c) * m + r] = a[c] * sh.D[c0 + c];
+        }
+    }
+  }
+}
+
+__device__ __forceinline__ void panel_tile(PanelTileShared& sh, const PanelItem it, int b,
+                                           const int32_t* __restrict__ col_primal, double* __restrict__ Lx, int64_t pt,
+                                           double* __restrict__ LDx, int64_t ldt, const double* __restrict__ anorm,
+                                           double pivot_eps, int* cnt) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, m = it.m, w = it.w;
+  double* P = Lx + b * pt + it.val;
+  double* PD = LDx + b * ldt + it.val;
+  for (int e = tid; e < kMaxSnWidth * kMaxSnWidth; e += kPanelThreads) {
+    const int c = e / kMaxSnWidth, r = e % kMaxSnWidth;
+    if (r < w && c <= r) sh.T[r][c] = P[(int64_t)c * m + r];
+    sh.U[c][r] = 0.0;
+  }
+  if (tid < kMaxSnWidth) sh.Di[tid] = 0.0;
+  __syncthreads();
+  if (it.factor) {
+    const double thr = pivot_eps * anorm[b];
+    for (int c = 0; c < w; c++) {
+      const double dv = panel_pivot(sh.T[c][c], thr, col_primal[it.first + c] != 0, cnt, tid == 0);
+      const double di = pivot_recip(dv);
+      if (tid < w - c - 1) {
+        const int r = c + 1 + tid;
+        const double lr = sh.T[r][c] * di;
+        sh.T[r][c] = lr;
+        sh.U[c][r] = lr * dv;
+      }
+      if (tid == 0) {
+        sh.D[c] = dv;
+        sh.Di[c] = di;
+      }
+      __syncthreads();
+      const int r = c + 1 + lane;
+      for (int c2 = c + 1 + warp; c2 < w; c2 += kPanelThreads / 32)
+        if (r >= c2 && r < w) sh.T[r][c2] -= sh.T[r][c] * sh.U[c][c2];
+      __syncthreads();
+    }
+    for (int e = tid; e < w * w; e += kPanelThreads) {
+      const int c = e / w, r = e - c * w;
+      const int64_t pos = (int64_t)c * m + r;
+      const double v = r == c ? sh.D[c] : (r > c ? sh.T[r][c] : P[pos]);
+      if (r >= c) P[pos] = v;
+      PD[pos] = v * sh.D[c];
+    }
+  } else {
+    if (tid < w) {
+      sh.D[tid] = sh.T[tid][tid];
+      sh.Di[tid] = pivot_recip(sh.T[tid][tid]);
+    }
+    for (int e = tid; e < w * w; e += kPanelThreads) {
+      const int c = e / w, r = e - c * w;
+      if (r > c) sh.U[c][r] = sh.T[r][c] * sh.T[c][c];
+    }
+    __syncthreads();
+  }
+  panel_rows(sh, P, PD, m, w, it.r0, it.r1);
+}
+
+__global__ void __launch_bounds__(kPanelThreads, 5)
+k_panel_factor(const SnDesc* __restrict__ small, int nsmall, int small_ctas, const PanelItem* __restrict__ items,
+               const int32_t* __restrict__ col_primal, double* __restrict__ Lx, int64_t pt, double* __restrict__ LDx,
+               int64_t ldt, const double* __restrict__ anorm, double pivot_eps, int N,
+               unsigned long long* __restrict__ counters) {
+  __shared__ union Shared {
+    __device__ Shared() {}
+    PanelSmallShared s;
+    PanelTileShared t;
+  } sh;
   __shared__ int cnt[4];
   if (threadIdx.x < 4) cnt[threadIdx.x] = 0;
-  for (int c = 0; c < w; c++) {
-    if (threadIdx.x == 0) {
-      double dv = P[(int64_t)c * m + c];
-      const bool primal = d.col_primal[f + c] != 0;
-      if (thr > 0.0 && fabs(dv) < thr) {
-        dv = primal ? thr : -thr;
-        cnt[3]++;
-      }
-      P[(int64_t)c * m + c] = dv;
-      cnt[dv > 0.0 ? 0 : (dv < 0.0 ? 1 : 2)]++;
-      dsh = dv;
-      dinv_sh = pivot_recip(dv);
-    }
-    __syncthreads();
-    const double dv = dsh, di = dinv_sh;
-    double* colc = P + (int64_t)c * m;
-    for (int r = c + 1 + threadIdx.x; r < m; r += blockDim.x) colc[r] = colc[r] * di;
-    __syncthreads();
-    for (int c2 = c + 1; c2 < w; c2++) {
-      const double l2 = colc[c2] * dv;
-      double* col2 = P + (int64_t)c2 * m;
-      for (int r = c2 + threadIdx.x; r < m; r += blockDim.x) col2[r] -= colc[r] * l2;
-    }
-    __syncthreads();
+  __syncthreads();
+  if ((int)blockIdx.x < small_ctas) {
+    panel_small(sh.s, small, nsmall, blockIdx.x, col_primal, Lx, pt, LDx, ldt, anorm, pivot_eps, N, cnt);
+  } else {
+    const int q = blockIdx.x - small_ctas;
+    panel_tile(sh.t, items[q / N], q % N, col_primal, Lx, pt, LDx, ldt, anorm, pivot_eps, cnt);
   }
+  __syncthreads();
   if (threadIdx.x < 4 && cnt[threadIdx.x]) atomicAdd(&counters[threadIdx.x], (unsigned long long)cnt[threadIdx.x]);
-  // L D of the panel for the updates of its ancestors: column c's entries
-  // times d_c, the product the updates would otherwise form per target tile
-  double* PD = LDx + b * ldt + d.sn_valoff[s];
-  for (int c = 0; c < w; c++) {
-    const double dv = P[(int64_t)c * m + c];
-    for (int r = threadIdx.x; r < m; r += blockDim.x) PD[(int64_t)c * m + r] = P[(int64_t)c * m + r] * dv;
-  }
 }
 
 }  // namespace
@@ -231,12 +384,16 @@ cudaError_t launch_factor_levels(Handle& h, cudaStream_t st) {
       kt_end(h, kt, st);
       h.launches++;
     }
-    const int s0 = h.flvl_ptr[l], s1 = h.flvl_ptr[l + 1];
-    if (s1 > s0) {
-      dim3 grid2(s1 - s0, h.N);
-      k_panel_factor<<<grid2, 256, 0, st>>>(h.d.flvl_sn + s0, h.d, h.Lx, pt, h.LDx, h.ld_total, h.anorm,
-                                            h.opt.pivot_eps,
-                                            h.counters);
+    // small panels and the triangles of the others, then the rows of the longest
+    const PanelLevel L = h.panel_lvl[l];
+    for (int second = 0; second < 2; second++) {
+      const int nsmall = second ? 0 : L.nsmall, nitem = second ? L.nrows : L.nitems;
+      const int64_t small_ctas = ((int64_t)nsmall * h.N + kPanelGroups - 1) / kPanelGroups;
+      const int64_t ctas = small_ctas + (int64_t)nitem * h.N;
+      if (ctas == 0) continue;
+      k_panel_factor<<<(unsigned)ctas, kPanelThreads, 0, st>>>(
+          h.d.panel_small + L.small0, nsmall, (int)small_ctas, h.d.panel_items + L.item0 + (second ? L.nitems : 0),
+          h.d.col_primal, h.Lx, pt, h.LDx, h.ld_total, h.anorm, h.opt.pivot_eps, h.N, h.counters);
       h.launches++;
     }
   }

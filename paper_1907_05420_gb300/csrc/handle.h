@@ -68,6 +68,20 @@ struct alignas(16) SnDesc {
   int32_t pad;
 };
 static_assert(sizeof(SnDesc) == 32, "SnDesc layout");
+// The block factor's panels: eight lanes take a panel of at most kPanelSmall
+// entries; a larger one has an item for its triangle and its rows or, with more
+// than kPanelRows rows below the triangle, for the triangle alone and one per
+// kPanelTile rows.  kPanelSmall: 16 panels stay within 16.5 KB per CTA.
+constexpr int kPanelSmall = 128, kPanelRows = 256, kPanelTile = 128;
+struct alignas(16) PanelItem {
+  int64_t val;                  // offset of the panel
+  int32_t first, w, m, r0, r1;  // first column, columns, rows; the rows [r0, r1) of the item
+  int32_t factor;               // 1: factors the triangle; 0: the triangle is factored
+};
+static_assert(sizeof(PanelItem) == 32, "PanelItem layout");
+struct PanelLevel {
+  int32_t small0 = 0, nsmall = 0, item0 = 0, nitems = 0, nrows = 0;  // items: nitems, then nrows for the second launch
+};
 // Supernodes that eight lanes solve with (at most this many columns and rows).
 constexpr int kSmallSnCols = 8, kSmallSnRows = 48;
 
@@ -118,13 +132,14 @@ struct DevSym {
   int32_t* g_rows = nullptr;       // W rows in contraction order: primal chunks, then multiplier chunks
   int32_t* trsv_jlo = nullptr;     // envelope of S (structured mode): first column block of each row block
   int32_t* trsv_jhi = nullptr;     // one past the last row block of each column block
-  SnDesc* flvl_desc = nullptr;     // the supernodes of flvl_sn
+  SnDesc* panel_small = nullptr;   // panels of at most kPanelSmall entries, by level (block factor)
+  PanelItem* panel_items = nullptr;  // items of the larger panels, by level
+  SnDesc* flvl_desc = nullptr;     // supernodes outside the dense tail, by level (solves)
   int64_t* fr_ptr = nullptr;       // per column: its row's records for the forward solve
   RowRec* fr_rec = nullptr;
   int32_t* wr_ptr = nullptr;       // per column of W: its nonzero rows outside the (augmented) tail
   int32_t* wr_row = nullptr;
   int32_t* w_sn = nullptr;         // per W row: its supernode
-  int32_t* flvl_sn = nullptr;      // supernodes outside the dense tail, by level (block factor)
   int32_t* twork = nullptr;        // tiles of the dense tail with updates from outside: 3 ints, tile row, tile column, first pair
   TailPair* tpairs = nullptr;
   int32_t* upd_ntail = nullptr;    // per supernode: leading updates from outside the tail
@@ -171,6 +186,7 @@ struct Handle {
   std::vector<int32_t> lvl_ptr;        // supernodes per level (host copy)
   std::vector<int32_t> reach_lvl_ptr;
   std::vector<int32_t> panel_rend;     // structured mode: per 64-wide panel, one past its last nonzero row
+  std::vector<PanelLevel> panel_lvl;   // the block factor's panels per level
   std::vector<int32_t> flvl_ptr;       // supernodes outside the dense tail per level (factor)
   std::vector<int32_t> flvl_small;     // and how many of them, the first ones, are small (kSmallSnCols, kSmallSnRows)
   int32_t nT = 0;                      // columns of the dense tail (0 = none)

@@ -168,7 +168,13 @@ struct PanelTileShared {
   double D[kMaxSnWidth], Di[kMaxSnWidth];  // d_c and 1 / d_c (0 from column w on)
 };
 
-// The pivot as it is used: a magnitude below thr becomes +-thr (thr > 0).  Bit
+// 0, which perturbs nothing, unless the product is positive (0 * Inf is not)
+__device__ __forceinline__ double panel_threshold(double pivot_eps, double anorm) {
+  const double thr = pivot_eps * anorm;
+  return thr > 0.0 ? thr : 0.0;
+}
+
+// The pivot as it is used: a magnitude below thr becomes +-thr (thr >= 0).  Bit
 // patterns of non-negative numbers order as the numbers do; a NaN stays.
 // cnt: positive, negative, zero or NaN, perturbed.
 __device__ __forceinline__ double panel_pivot(double dv, double thr, bool primal, int* cnt, bool count) {
@@ -198,7 +204,7 @@ __device__ __forceinline__ void panel_small(PanelSmallShared& sh, const SnDesc* 
   double* T = sh.t[g];
   double* P = Lx + b * pt + S.val;
   double* PD = LDx + b * ldt + S.val;
-  const double thr = on ? pivot_eps * anorm[b] : 0.0;
+  const double thr = on ? panel_threshold(pivot_eps, anorm[b]) : 0.0;
   for (int e = l; e < w * m; e += 8) T[e] = P[e];
   const int wmax = __reduce_max_sync(0xffffffffu, w);
   __syncwarp();
@@ -278,7 +284,7 @@ __device__ __forceinline__ void panel_tile(PanelTileShared& sh, const PanelItem 
   if (tid < kMaxSnWidth) sh.Di[tid] = 0.0;
   __syncthreads();
   if (it.factor) {
-    const double thr = pivot_eps * anorm[b];
+    const double thr = panel_threshold(pivot_eps, anorm[b]);
     for (int c = 0; c < w; c++) {
       const double dv = panel_pivot(sh.T[c][c], thr, col_primal[it.first + c] != 0, cnt, tid == 0);
       const double di = pivot_recip(dv);

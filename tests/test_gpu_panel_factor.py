@@ -46,3 +46,25 @@ def test_panels_match_dense_tail(spec, prec):
         counts.append([info[k] for k in ("n_pos", "n_neg", "n_zero", "n_perturbed")])
     assert np.max(np.abs(xs[0] - xs[1])) <= 1e-9 * np.max(np.abs(xs[1]))
     assert counts[0] == counts[1]
+
+
+@pytest.mark.parametrize("spec", [CONFIGS["tiny"], GridSpec(301, 411, 40, 13, 3, 1e-3, 1e3, 5)],
+                         ids=lambda s: f"{s.n_bus}x{s.n_per}")
+def test_threshold_that_is_not_positive(spec):
+    """pivot_eps = 0 turns the perturbation off, also where max|A_i| is infinite
+    (0 * Inf is no threshold)."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1907_05420_gb300 import binding as B
+
+    p = make_problem(spec)
+    a = np.array(p.a_vals, dtype=np.float64).reshape(p.N, -1)
+    a[0, 0] = np.inf
+    for tail in (0, 1):
+        h = B.kkt_analyze(p, B.kkt_default_options("fp64", pivot_eps=0.0, dense_tail=tail))
+        try:
+            B.kkt_factor(h, a, np.ascontiguousarray(p.b_vals), np.ascontiguousarray(p.c_vals))
+            assert B.kkt_get_info(h)["n_perturbed"] == 0
+        finally:
+            B.kkt_destroy(h)

@@ -519,9 +519,10 @@ kkt_status kkt_server_cache_info(kkt_server* s, int64_t* resident, int64_t* anal
  * update of S with 256-wide outer panels (k_tc_update_wide), 2 the 64-wide
  * TF32/BF16 update (k_tc_update), 3 the FP64 dense update on the CUDA cores
  * (k_dense_update: S in KKT_FP64, the FP64 tails), 4 the supernodal updates of
- * the block factor (k_factor_update), 5 the dense diagonal blocks of the
+ * the block factor (k_factor_update, k_tail_update), 5 the dense diagonal blocks of the
  * blocked factors (k_dense_diag_t), 6 the emulated-FP64 update with K = 256
- * of the 256-wide outer panels (k_tc_update_emu_wide), 7 the emulated-FP64
+ * of the 256-wide outer panels and the tails' update by their heavy
+ * descendants (k_tc_update_emu_wide), 7 the emulated-FP64
  * panels of those factors (k_tc_panel_emu, timed with the launch that forms
  * its operands: W = L11^{-1} and the digit images of W and A21).  flops: the
  * algorithmic FP64-equivalent flops of the launches (2 per multiply-add on the

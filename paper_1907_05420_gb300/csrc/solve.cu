@@ -3,12 +3,12 @@
 // iterative refinement on the full K.
 //
 // One application of the factored K^{-1} to r = [r_0..r_{N-1}; r_g]:
-//   z_i = L_i^{-1} P^T r_i                       (k_fsolve_level, level by level)
+//   z_i = L_i^{-1} P^T r_i                       (k_fsolve_lvl, level by level)
 //   u_i = W_i^T D_i^{-1} z_i                     (k_reduce_u: E^T A_i^{-1} r_i)
 //   t   = r_g - sum_i M_i^T u_i                  (k_reduce_t, block order)
 //   x_g = S^{-1} t                               (dense solve)
 //   z_i -= W_i (M_i x_g)                         (k_apply_xg: L^{-1} P^T B_i x_g)
-//   x_i = P L_i^{-T} D_i^{-1} z_i                (k_diag_scale, k_bsolve_level)
+//   x_i = P L_i^{-T} D_i^{-1} z_i                (k_diag_scale, k_bsolve_lvl)
 // which is x_i = A_i^{-1} (r_i - B_i x_g).  Every output is summed by one thread
 // or one warp in a fixed order.
 #include "handle.h"

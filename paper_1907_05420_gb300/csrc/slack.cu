@@ -37,6 +37,10 @@ namespace {
 // The divisions keep the FP64 pipe busy and the copy the memory, so one launch
 // that does both overlaps them (2,383 buses x 96 periods, 20 million values read
 // and written or read: 44 us, where the copies took 22 us and the rows 37 us).
+// The off-diagonal entries of a dense C are copied by the whole grid, a row per
+// CTA at a time: orders 289, 1,000, 2,000 and 4,000 take 13, 13, 23 and 52 us in
+// all (24, 30, 32 and 63 with device copies of A and C before the rows, 19, 117,
+// 345 and 1,097 with C left to the CTAs of the coupling rows).
 template <bool COPY_A>
 __global__ void __launch_bounds__(256, 5)
 k_slack_reduce(const int32_t* __restrict__ diag_pos, const int32_t* __restrict__ ineq_of_row,
@@ -50,6 +54,24 @@ k_slack_reduce(const int32_t* __restrict__ diag_pos, const int32_t* __restrict__
                double* a_vals, double* c_vals, double* __restrict__ rhs) {
   constexpr int kInFlight = 8;
   const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = gridDim.x * (int64_t)blockDim.x;
+  if (copy_c)
+    for (int64_t c = blockIdx.y * (int64_t)gridDim.x + blockIdx.x; c < nC; c += (int64_t)gridDim.x * gridDim.y) {
+      const double* src = c_base + c * nC;
+      double* dst = c_vals + c * nC;
+      for (int i0 = threadIdx.x; i0 < nC; i0 += kInFlight * blockDim.x) {
+        double v[kInFlight];
+#pragma unroll
+        for (int u = 0; u < kInFlight; u++) {
+          const int i = i0 + u * blockDim.x;
+          if (i < nC) v[u] = src[i];
+        }
+#pragma unroll
+        for (int u = 0; u < kInFlight; u++) {
+          const int i = i0 + u * blockDim.x;
+          if (i < nC && i != c) dst[i] = v[u];
+        }
+      }
+    }
   for (int64_t b = blockIdx.y; b <= N; b += gridDim.y) {
     const bool border = b == N;
     if (COPY_A && !border) {
@@ -72,9 +94,6 @@ k_slack_reduce(const int32_t* __restrict__ diag_pos, const int32_t* __restrict__
         }
       }
     }
-    if (border && copy_c)
-      for (int64_t i = t0; i < (int64_t)nC * nC; i += step)
-        if (i % (nC + 1) != 0) c_vals[i] = c_base[i];
     const int rows = border ? nC : nA;
     for (int64_t r = t0; r < rows; r += step) {
       const int64_t q = b * nA + r;
@@ -200,10 +219,12 @@ kkt_status kkt_slack_reduce(kkt_slack* sl, const kkt_ipm_state* st, const double
   (void)cudaGetLastError();
   // the entries other than the diagonals keep their base values (a diagonal C has none)
   const int copy_c = c_vals != c_base && h.c_kind != 0;
-  const dim3 grid(grid_of(std::max(h.nA, h.nC)), std::min(h.N + 1, 65535));
-  (a_vals != a_base ? k_slack_reduce<true> : k_slack_reduce<false>)<<<grid, 256, 0, s>>>(h.d.diag_pos, sl->ineq_of_row, sl->diag_mask, h.nA, h.nP, h.N, h.nC, sl->L,
-                                      h.nnzA, h.c_kind, copy_c, st->x, st->z, st->s, st->y, st->la, st->le,
-                                      st->lcd, st->lb, st->lf, a_base, c_base, a_vals, c_vals, rhs);
+  dim3 grid(grid_of(std::max(h.nA, h.nC)), std::min(h.N + 1, 65535));
+  // the rows of C spread over all CTAs, five of which fit an SM
+  if (copy_c) grid.x = std::max(grid.x, (std::min(h.nC, 152 * 5) + grid.y - 1) / grid.y);
+  (a_vals != a_base ? k_slack_reduce<true> : k_slack_reduce<false>)<<<grid, 256, 0, s>>>(
+      h.d.diag_pos, sl->ineq_of_row, sl->diag_mask, h.nA, h.nP, h.N, h.nC, sl->L, h.nnzA, h.c_kind, copy_c, st->x,
+      st->z, st->s, st->y, st->la, st->le, st->lcd, st->lb, st->lf, a_base, c_base, a_vals, c_vals, rhs);
   h.launches++;
   KKT_CUDA(cudaGetLastError());
   return KKT_OK;

@@ -30,8 +30,10 @@ kkt_symbolic* kkt_symbolic_create(int32_t nA, int32_t nP, const int32_t* a_rowpt
  * panel_rend, jlo, jhi, colcount, upd_ntail, stats (n, nsuper, nlevels,
  * panel_total, nnzL, k, nw, tail_sn, tail_col, nw_before_tail), tail_wrow
  * (per tail column its W row, -1 outside the reach), wt_ptr / wt_idx (per
- * supernode the columns of W that are nonzero on it).  The dense tail is
- * chosen as kkt_analyze chooses it with the dense_tail option on. */
+ * supernode the columns of W that are nonzero on it), heavy (the supernodes
+ * whose updates of the dense tail the emulated tail of at least 512 columns
+ * takes as one product).  The dense tail is chosen as kkt_analyze chooses it
+ * with the dense_tail option on. */
 int64_t kkt_symbolic_get(const kkt_symbolic* sym, const char* name, int64_t* out);
 
 /* Re-chooses the dense tail with cost ratio `ratio` and the byte cap

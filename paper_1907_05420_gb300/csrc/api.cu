@@ -69,7 +69,7 @@ void free_all(Handle* h) {
                   h->c_vals, h->anorm, h->W, h->G, h->S, h->Ypanel, h->knorm, h->counters, h->r,
                   h->z, h->u, h->v, h->tg, h->xg, h->x, h->dx, h->rho, h->rhs, h->red,
                   h->Zs, h->trsv_s, h->trsv_t, h->dev_err, h->S32, h->Y32, h->tw_img, h->ew_s_Y, h->ew_s_A,
-                  h->ew_s_B, h->ew_s_scale, h->ew_t_Y, h->ew_t_A, h->ew_t_B, h->ew_t_scale, h->tc_imgA,
+                  h->ew_s_B, h->ew_s_scale, h->ew_t_Y, h->ew_t_A, h->ew_t_B, h->ew_t_scale, h->hv_bad, h->tc_imgA,
                   h->tc_imgB, h->tc_scaleA, h->tc_scaleB, h->gm_V, h->gm_Z, h->d.cum_y_ptr, h->d.cum_y_t,
                   h->d.cum_y_e, h->d.cum_z_ptr, h->d.cum_z_t, h->d.cum_z_e, h->d.cum_check, h->cum_err,
                   h->rstate, h->cum_Q32, h->cum_QY32, h->cum_Linv32, h->cum_M32, h->cum_Mt32, h->cum_D32, h->cum_H, h->cum_Sd, h->cum_So, h->cum_Q, h->cum_QY, h->cum_Linv, h->cum_M, h->cum_Mt,
@@ -840,6 +840,7 @@ kkt_status analyze_one(const kkt_pattern* pat, const kkt_options* opt, double ta
       AL(ew_t_A, uint8_t, emu_wide_image_bytes(h->nTa) * h->N);
       AL(ew_t_B, uint8_t, emu_wide_image_bytes(h->nTa) * h->N);
       AL(ew_t_scale, double, 2 * ((int64_t)h->nTa + 256) * h->N);
+      if (h->hv_cols > 0) AL(hv_bad, int, h->N);
     }
   }
   AL(knorm, double, 1);

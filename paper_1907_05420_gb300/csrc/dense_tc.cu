@@ -1151,7 +1151,7 @@ __global__ void __launch_bounds__(256, 2) k_slice_heavy(const double* __restrict
                                                      int ncol, int nT, int mpad, uint8_t* __restrict__ imgA0,
                                                      uint8_t* __restrict__ imgB0, double* __restrict__ scaleA0,
                                                      double* __restrict__ scaleB0, int64_t img_stride,
-                                                     int64_t scale_stride) {
+                                                     int64_t scale_stride, int* __restrict__ bad) {
   __shared__ unsigned long long mx[8][32];
   __shared__ uint32_t bf16_of_byte[256];
   const int64_t bb = blockIdx.y;
@@ -1179,9 +1179,39 @@ __global__ void __launch_bounds__(256, 2) k_slice_heavy(const double* __restrict
 #pragma unroll
   for (int e = 0; e < kEwWarpCols; e++) mag = max(mag, magnitude_bits(v[e]));
   mag = max_over_warps(mag, mx);  // (its barrier covers the table too)
+  if (mag >= kInfBits) bad[bb] = 1;
   const int e_exp = mag ? scale_exponent(mag) + 1 : 0;  // |v| < 2^(e-1)
   if (k == 0) (isA ? scaleA0 : scaleB0)[bb * scale_stride + rho] = ldexp(1.0, e_exp);
   slice_columns(v, e_exp, (isA ? imgA0 : imgB0) + bb * img_stride, rho, isA, k, bf16_of_byte);
+}
+
+// The heavy update of the matrices with a NaN or an Inf in a heavy panel, in
+// FP64: digits of such a value are finite, and the tail's pivots would no longer
+// show it.  Entry by entry over the columns that have both rows, as the
+// supernodal updates run; a matrix of finite panels costs a look at its flag (24
+// blocks of 9,241 buses: a step 165.0 ms before, 165.1 with it).
+__global__ void __launch_bounds__(256) k_heavy_nonfinite(const int* __restrict__ bad, int N,
+                                                         const double* __restrict__ Lx, int64_t pt,
+                                                         const double* __restrict__ LDx, int64_t ldt,
+                                                         const int64_t* __restrict__ off,
+                                                         const int32_t* __restrict__ sn,
+                                                         const int32_t* __restrict__ pos, int ncol, int nT,
+                                                         double* __restrict__ T, int nTa) {
+  for (int b = 0; b < N; b++) {
+    if (!bad[b]) continue;
+    const double* L = Lx + b * pt;
+    const double* LD = LDx + b * ldt;
+    double* Tb = T + (int64_t)b * nTa * nTa;
+    for (int64_t j = blockIdx.x; j < nT; j += gridDim.x)
+      for (int64_t i = j + threadIdx.x; i < nT; i += blockDim.x) {
+        double acc = 0.0;
+        for (int c = 0; c < ncol; c++) {
+          const int32_t* p = pos + (int64_t)sn[c] * nT;
+          if (p[i] >= 0 && p[j] >= 0) acc += L[off[c] + p[i]] * LD[off[c] + p[j]];
+        }
+        Tb[i + j * nTa] -= acc;
+      }
+  }
 }
 
 // The K = 256 emulated update: one CTA per run of up to kEmuRun tiles (I, J)
@@ -1196,7 +1226,8 @@ __global__ void __launch_bounds__(kEmuThreads, 1)
     k_tc_update_emu_wide(double* __restrict__ S0, int n, int base, int m, int TI, int TJ, int jmode, int nchunk,
                          const uint8_t* __restrict__ imgA0, const uint8_t* __restrict__ imgB0,
                          const double* __restrict__ scaleA0, const double* __restrict__ scaleB0,
-                         int64_t s_stride, int64_t img_stride, int64_t scale_stride, int* err) {
+                         int64_t s_stride, int64_t img_stride, int64_t scale_stride, const int* skip, int* err) {
+  if (skip && skip[blockIdx.y]) return;  // (the heavy update: k_heavy_nonfinite's matrices)
   constexpr uint32_t TMEM_COLS = 512;  // 7 levels x 64 columns
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ __align__(8) uint64_t bar_full[kEwStages], bar_empty[kEwStages], bar_tfull, bar_tempty;
@@ -1838,7 +1869,7 @@ cudaError_t factor_emu_wide(Handle& h, double* S, int n, int npiv, int nb, const
       const cudaError_t le = launch_prio(k_tc_update_emu_wide, dim3(tasks, nb), dim3(kEmuThreads), ew_smem_bytes(),
                                          us, uprio, S, n, base, m, TI, TJ, jmode, nchunk, (const uint8_t*)ew.A,
                                          (const uint8_t*)ew.B, (const double*)ew.sA, (const double*)ew.sB, ts.s,
-                                         ew.img_stride, ew.scale_stride, h.dev_err);
+                                         ew.img_stride, ew.scale_stride, (const int*)nullptr, h.dev_err);
       kt_end(h, kt, us);
       return le;
     };
@@ -2057,17 +2088,21 @@ cudaError_t launch_tail_heavy_update(Handle& h, cudaStream_t st) {
   const int TI = (nT + TM - 1) / TM, TJ = (nT + TN - 1) / TN, mpad = TI * TM;
   const int64_t is = emu_wide_image_bytes(nTa), ss = 2 * ((int64_t)nTa + 2 * TM);
   double *sA = h.ew_t_scale, *sB = h.ew_t_scale + (nTa + 2 * TM);
+  cudaError_t e = cudaMemsetAsync(h.hv_bad, 0, sizeof(int) * N, st);
+  if (e != cudaSuccess) return e;
   k_slice_heavy<<<dim3(2 * mpad / 32, N), 256, 0, st>>>(h.Lx, h.sym.panel_total, h.LDx, h.ld_total, h.d.hv_off,
                                                         h.d.hv_sn, h.d.hv_col, h.d.hv_pos, h.hv_cols, nT, mpad,
-                                                        h.ew_t_A, h.ew_t_B, sA, sB, is, ss);
+                                                        h.ew_t_A, h.ew_t_B, sA, sB, is, ss, h.hv_bad);
   int tasks = 0;
   for (int I = 0; I < TI; I++) tasks += emu_row_tasks(I, TJ, 0, 4);
   const int kt = kt_begin(h, kFamEmuWide, N * update_flops(nT, 0, nT, h.hv_cols), st);
   k_tc_update_emu_wide<<<dim3(tasks, N), kEmuThreads, ew_smem_bytes(), st>>>(
       h.Tt, nTa, 0, nT, TI, TJ, 0, (h.hv_cols + kEwChunk - 1) / kEwChunk, h.ew_t_A, h.ew_t_B, sA, sB,
-      (int64_t)nTa * nTa, is, ss, h.dev_err);
+      (int64_t)nTa * nTa, is, ss, h.hv_bad, h.dev_err);
   kt_end(h, kt, st);
-  h.launches += 2;
+  k_heavy_nonfinite<<<152 * 8, 256, 0, st>>>(h.hv_bad, N, h.Lx, h.sym.panel_total, h.LDx, h.ld_total, h.d.hv_off,
+                                             h.d.hv_sn, h.d.hv_pos, h.hv_cols, nT, h.Tt, nTa);
+  h.launches += 3;
   return cudaGetLastError();
 }
 

@@ -123,6 +123,8 @@ KKT_HD int exp_field(double v) { return (int)((bits_of(v) >> 52) & 0x7FF); }
 // largest one is found without the FP64 pipe.
 KKT_HD unsigned long long magnitude_bits(double v) { return (unsigned long long)bits_of(v) & 0x7FFFFFFFFFFFFFFFull; }
 
+constexpr unsigned long long kInfBits = 0x7FF0000000000000ull;  // magnitude bits of Inf; a NaN's are larger
+
 // The exponent e with 2^(e-1) <= |v| < 2^e of the magnitude with these bits
 // (normal or subnormal; 0 for zero).
 KKT_HD int scale_exponent(unsigned long long mag) {

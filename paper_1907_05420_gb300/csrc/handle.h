@@ -200,6 +200,7 @@ struct Handle {
   std::vector<int32_t> reach_lvl_chunks, reach_lvl_chunks_nt;  // W solve: 32-column chunks per level
   int64_t g_nkeys = 0;                 // nonzero entries of the sparse contraction
   int32_t hv_cols = 0;                 // columns of the tail's heavy descendants (0: none)
+  int* hv_bad = nullptr;               // N: whether a heavy panel holds a NaN or an Inf
   int32_t tail_items = 0;              // tiles of the dense tail in d.twork
   std::vector<double> fupd_flops;      // algorithmic flops of one block's supernodal updates, per level
   double tupd_flops = 0.0;             // and of the tail's updates from outside it
@@ -366,7 +367,6 @@ cudaError_t launch_factor_levels(Handle& h, cudaStream_t st);
 cudaError_t launch_dense_tail(Handle& h, cudaStream_t st);
 cudaError_t launch_tail_factor_emulated(Handle& h, cudaStream_t st);  // (dense_tc.cu)
 cudaError_t launch_tail_heavy_update(Handle& h, cudaStream_t st);     // (dense_tc.cu)
-constexpr int kHeavyMaxCols = 256;  // K of the 256-wide emulated update
 // ---- (schur.cu) ----
 cudaError_t launch_w_solve(Handle& h, cudaStream_t st);
 cudaError_t launch_w_solve_before_tail(Handle& h, cudaStream_t st);

@@ -86,6 +86,7 @@ void choose_tail(Symbolic& S, int32_t N, int64_t max_bytes, int32_t min_cols, do
 // replace.  At most max_cols columns in all (the ones with the most rows
 // first); returned in increasing order, empty if there is nothing to gain.
 std::vector<int32_t> heavy_descendants(const Symbolic& S, int32_t max_cols);
+constexpr int32_t kHeavyMaxCols = 256;  // K of the 256-wide emulated update
 
 // Coupling analysis: B_i (COO per block) against the block factor.
 // With E the sorted union of the rows that carry a nonzero of some B_i

@@ -77,6 +77,7 @@ int64_t kkt_symbolic_get(const kkt_symbolic* sym, const char* name, int64_t* out
   if (n == "wt_ptr") return copy_out(C.wt_ptr, out);
   if (n == "wt_idx") return copy_out(C.wt_idx, out);
   if (n == "upd_ntail") return copy_out(S.upd_ntail, out);
+  if (n == "heavy") return copy_out(kkt::heavy_descendants(S, kkt::kHeavyMaxCols), out);
   if (n == "tail_wrow") {
     std::vector<int32_t> tw;
     kkt::tail_w_rows(S, C, tw);

@@ -45,7 +45,8 @@ typedef enum {
   KKT_ERR_ZERO_PIVOT = 4,    /* a pivot was exactly zero and pivot_eps is 0 */
   KKT_ERR_INERTIA = 5,       /* inertia differs from (N*nP + nC, N*(nA-nP), 0) */
   KKT_ERR_NOT_CONVERGED = 6, /* refinement did not reach refine_tol */
-  KKT_ERR_TIMEOUT = 7,       /* a bounded device wait ran out */
+  KKT_ERR_TIMEOUT = 7,       /* a bounded device wait ran out: nothing computed since the handle's
+                                last factorization is valid; the next one clears the condition */
   KKT_ERR_STATE = 8,         /* call out of order (e.g. solve before factor) */
   KKT_ERR_NONFINITE = 9      /* a NaN or Inf in the values of K or the right-hand side, or a
                                 solution that is not finite after the FP64 fallback */
@@ -413,7 +414,9 @@ kkt_status kkt_residual(kkt_handle* h, const double* rhs, const double* x, doubl
  * coupling rows hold sum |B column| + sum |C row| over the handle's blocks. */
 kkt_status kkt_abs_rowsums(kkt_handle* h, double* out, void* stream);
 /* *out = max |v_i| over n device doubles (NaN if any entry is NaN);
- * synchronizes `stream`. */
+ * synchronizes `stream`.  KKT_ERR_TIMEOUT if a bounded device wait of the
+ * handle has run out since its last factorization: the call of the sequence
+ * that reports it, as the others do not wait for the device. */
 kkt_status kkt_norm_inf(kkt_handle* h, const double* v, int64_t n, double* out, void* stream);
 
 /* ---- slack elimination around the solve (Sec. 2, eqs. SCOPFhessian,
@@ -548,6 +551,10 @@ kkt_status kkt_measure_fp64_peak(double* gflops);
  * 1.0 / d[i] by CUDA's FP64 division, so that tests can bound the
  * difference.  Device arrays; asynchronous on `stream`. */
 kkt_status kkt_probe_pivot_reciprocal(const double* d, int64_t n, double* recip, double* quotient, void* stream);
+
+/* Diagnostic: leaves the handle as a bounded device wait that runs out on
+ * `stream` leaves it, so that tests see what the calls after it report. */
+kkt_status kkt_probe_wait_expired(kkt_handle* h, void* stream);
 
 #ifdef __cplusplus
 }

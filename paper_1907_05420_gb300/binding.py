@@ -84,7 +84,7 @@ EXPORTS = ["kkt_default_options", "kkt_analyze", "kkt_factor", "kkt_solve", "kkt
            "kkt_solve_front", "kkt_solve_coupling", "kkt_solve_back", "kkt_residual", "kkt_abs_rowsums",
            "kkt_norm_inf", "kkt_kernel_stats", "kkt_slack_create", "kkt_slack_reduce", "kkt_slack_recover",
            "kkt_slack_destroy", "kkt_server_set_cache", "kkt_server_submit_pattern", "kkt_server_cache_info",
-           "kkt_schur_blocks", "kkt_probe_pivot_reciprocal"]
+           "kkt_schur_blocks", "kkt_probe_pivot_reciprocal", "kkt_probe_wait_expired"]
 
 KERNEL_FAMILIES = ["k_tc_update_emu", "k_tc_update_wide", "k_tc_update", "k_dense_update", "k_factor_update",
                    "k_dense_diag_t", "k_tc_update_emu_wide", "k_tc_panel_emu"]
@@ -161,6 +161,7 @@ def load(build_if_missing: bool = True):
                        ("kkt_schur_factor_copy", [vp, vp, vp]),
                        ("kkt_schur_blocks", [vp, vp, vp, vp]),
                        ("kkt_probe_pivot_reciprocal", [vp, C.c_int64, vp, vp, vp]),
+                       ("kkt_probe_wait_expired", [vp, vp]),
                        ("kkt_accumulate", [vp, C.c_int64, vp, C.c_int64, C.c_int64, C.c_int64, vp]),
                        ("kkt_solve_front", [vp, vp, vp, vp]),
                        ("kkt_solve_coupling", [vp, vp, vp, vp]),
@@ -439,6 +440,11 @@ def kkt_probe_pivot_reciprocal(d, recip, quotient, stream=None):
     """recip = the factor kernels' pivot reciprocal of d, quotient = 1.0 / d (device tensors)."""
     return _check(load().kkt_probe_pivot_reciprocal(_dev(d), int(d.numel()), _dev(recip), _dev(quotient),
                                                     _stream_ptr(stream)))
+
+
+def kkt_probe_wait_expired(h, stream=None):
+    """Leaves the handle as a bounded device wait that ran out does."""
+    return _check(load().kkt_probe_wait_expired(h, _stream_ptr(stream)))
 
 
 def kkt_accumulate(dst_ptr, ld_dst, src, ld_src, rows, cols, stream=None):

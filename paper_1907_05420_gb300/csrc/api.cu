@@ -68,7 +68,7 @@ void free_all(Handle* h) {
                   h->t_scaleA, h->t_scaleB, h->Lx, h->LDx, h->a_vals, h->b_vals,
                   h->c_vals, h->anorm, h->W, h->G, h->S, h->Ypanel, h->knorm, h->counters, h->r,
                   h->z, h->u, h->v, h->tg, h->xg, h->x, h->dx, h->rho, h->rhs, h->red,
-                  h->Zs, h->trsv_s, h->trsv_t, h->dev_err, h->S32, h->Y32, h->tw_img, h->ew_s_Y, h->ew_s_A,
+                  h->Zs, h->trsv_s, h->trsv_t, h->S32, h->Y32, h->tw_img, h->ew_s_Y, h->ew_s_A,
                   h->ew_s_B, h->ew_s_scale, h->ew_t_Y, h->ew_t_A, h->ew_t_B, h->ew_t_scale, h->hv_bad, h->tc_imgA,
                   h->tc_imgB, h->tc_scaleA, h->tc_scaleB, h->gm_V, h->gm_Z, h->d.cum_y_ptr, h->d.cum_y_t,
                   h->d.cum_y_e, h->d.cum_z_ptr, h->d.cum_z_t, h->d.cum_z_e, h->d.cum_check, h->cum_err,
@@ -107,7 +107,7 @@ cudaError_t record(Handle& h, cudaEvent_t ev, cudaStream_t st) {
 // as a CUDA graph and replayed.
 cudaError_t enqueue_factor(Handle& h, cudaStream_t st, bool with_s = true) {
   h.kt_used = 0;
-  cudaError_t e = cudaMemsetAsync(h.counters, 0, sizeof(unsigned long long) * 2 * kNumCounters, st);
+  cudaError_t e = cudaMemsetAsync(h.counters, 0, sizeof(unsigned long long) * (2 * kNumCounters + 1), st);
 #define STEP(x) \
   if (e == cudaSuccess) e = (x)
   STEP(launch_scatter_a(h, st));
@@ -844,7 +844,8 @@ kkt_status analyze_one(const kkt_pattern* pat, const kkt_options* opt, double ta
     }
   }
   AL(knorm, double, 1);
-  AL(counters, unsigned long long, 2 * kNumCounters);  // second half: discarded counts
+  AL(counters, unsigned long long, 2 * kNumCounters + 1);
+  h->dev_err = reinterpret_cast<int*>(h->counters + 2 * kNumCounters);
   AL(z, double, (int64_t)h->N * n);
   AL(u, double, k * h->N);
   AL(v, double, k * h->N);
@@ -892,7 +893,6 @@ kkt_status analyze_one(const kkt_pattern* pat, const kkt_options* opt, double ta
       AL(ew_s_scale, double, 2 * ((int64_t)h->nC + 256));
     }
   }
-  AL(dev_err, int, 1);
 #undef AL
   if (e == cudaSuccess) e = cudaMemset(h->dev_err, 0, sizeof(int));
   // W's structurally zero entries are never written: clear it once

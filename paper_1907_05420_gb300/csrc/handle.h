@@ -248,7 +248,7 @@ struct Handle {
   bool g_reduced = false;     // S assembled from a TF32/BF16 contraction
   int g_nchunks = 0, g_nchunks_pos = 0;  // 64-row chunks of g_rows (positive-pivot chunks first)
   double* knorm = nullptr;    // ||K||_inf
-  unsigned long long* counters = nullptr;  // kNumCounters
+  unsigned long long* counters = nullptr;  // 2 kNumCounters; dev_err behind them, cleared with them by every factor
   // solve work vectors
   double* r = nullptr;        // nK: right-hand side being solved
   double* z = nullptr;        // N * nA
@@ -267,7 +267,7 @@ struct Handle {
   double* Zs = nullptr;       // 2 * ceil(nC/64) * 64 * 64: products that the solves with S fuse (dense.cu)
   double* trsv_s = nullptr;   // publishing vectors and tickets of the dense triangular solves: of S
   double* trsv_t = nullptr;   // and of the tails
-  int* dev_err = nullptr;     // set when a bounded device wait runs out
+  int* dev_err = nullptr;     // set when a bounded device wait runs out, until the next factorization
   // device-side refinement (opt.device_refine): the solve graph and its loop state
   // (eta, eta_prev, steps, outcome: 0 converged, 1 stopped above the tolerance, 2 not finite)
   // one graph per kind of factor of S (s_factor: the FP32 one of the TF32/BF16

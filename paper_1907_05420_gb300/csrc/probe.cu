@@ -52,6 +52,17 @@ extern "C" kkt_status kkt_probe_pivot_reciprocal(const double* d, int64_t n, dou
   return KKT_OK;
 }
 
+extern "C" kkt_status kkt_probe_wait_expired(kkt_handle* hh, void* stream) {
+  using namespace kkt;
+  Handle* h = reinterpret_cast<Handle*>(hh);
+  if (!h) {
+    set_error("kkt_probe_wait_expired: null handle");
+    return KKT_ERR_INVALID;
+  }
+  KKT_CUDA(cudaMemsetAsync(h->dev_err, 1, sizeof(int), (cudaStream_t)stream));
+  return KKT_OK;
+}
+
 extern "C" kkt_status kkt_measure_fp64_peak(double* gflops) {
   using namespace kkt;
   if (!gflops) return KKT_ERR_INVALID;

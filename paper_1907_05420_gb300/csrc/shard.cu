@@ -100,6 +100,12 @@ __global__ void k_maxabs(const double* __restrict__ v, int64_t n, double* __rest
     atomicMax(reinterpret_cast<unsigned long long*>(out), (unsigned long long)__double_as_longlong(sh[0]));
 }
 
+// The norm and the handle's error flag, straight into pinned host memory.
+__global__ void k_publish_norm(const double* __restrict__ norm, const int* __restrict__ dev_err, double* host) {
+  if (threadIdx.x == 0) host[5] = *norm;
+  if (threadIdx.x == 1) *reinterpret_cast<int*>(host + 4) = *dev_err;
+}
+
 __global__ void k_f32_to_f64(const float* __restrict__ a, double* __restrict__ b, int64_t n) {
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x)
     b[q] = (double)a[q];
@@ -313,8 +319,14 @@ kkt_status kkt_norm_inf(kkt_handle* hh, const double* v, int64_t n, double* out,
     k_maxabs<<<grid_of(n), 256, 0, st>>>(v, n, h->red + 8);
     h->launches++;
   }
-  KKT_CUDA(cudaMemcpyAsync(h->host_red + 5, h->red + 8, sizeof(double), cudaMemcpyDeviceToHost, st));
+  k_publish_norm<<<1, 32, 0, st>>>(h->red + 8, h->dev_err, h->host_red);
+  h->launches++;
+  KKT_CUDA(cudaGetLastError());
   KKT_CUDA(cudaStreamSynchronize(st));
+  if (*reinterpret_cast<int*>(h->host_red + 4) != 0) {
+    set_error("kkt_norm_inf: a bounded device wait ran out in an earlier call on this handle");
+    return KKT_ERR_TIMEOUT;
+  }
   *out = h->host_red[5];
   return KKT_OK;
 }

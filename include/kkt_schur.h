@@ -101,9 +101,11 @@ typedef struct {
                           with the expected sign and counted; 0 turns the perturbation off */
   int32_t use_graphs;  /* capture the device work of kkt_factor after the input copies as a CUDA
                           graph at the handle's first kkt_factor and replay it on later calls.
-                          kkt_solve's application of the factorization and its refinement steps
-                          launch directly the first time and become graphs at the second (per
-                          kind of factor of S; not a GMRES cycle).  Default 1. */
+                          kkt_solve's application of the factorization becomes a graph at the end
+                          of that kkt_factor, on the host while the device runs the factor (with
+                          early_solve at the second use), and its refinement step at the second
+                          use, which costs that call some 100 us on the host (per kind of factor
+                          of S; not a GMRES cycle).  Default 1. */
   int32_t fp64_fallback; /* refactor S in FP64 when refinement stalls in a reduced mode */
   int32_t reduced_contraction; /* KKT_TF32/KKT_BF16 only: also run the Schur contraction
                                   G_i = W_i^T D_i^{-1} W_i on the tensor cores in that precision

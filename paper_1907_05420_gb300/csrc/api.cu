@@ -970,6 +970,62 @@ double time_factor(kkt_handle* hh, const kkt_pattern* pat) {
   return ms;
 }
 
+// kkt_solve's host loop up to its next look at the norms: the application of
+// the factorization to h.rhs into h.x, or with `refine` to the residual and x +=
+// dx; then the residual, its norms and what the test reads.
+cudaError_t enqueue_apply(Handle& h, bool refine, cudaStream_t st) {
+  cudaError_t e = refine ? launch_apply_inverse(h, h.rho, h.dx, st) : launch_apply_inverse(h, h.rhs, h.x, st);
+  if (e == cudaSuccess && refine) e = launch_axpy(h, h.x, h.dx, (int64_t)h.N * h.nA + h.nC, st);
+  if (e == cudaSuccess) e = launch_residual(h, h.rhs, h.x, h.rho, st);
+  if (e == cudaSuccess) e = launch_norms(h, h.rho, h.x, h.rhs, st);
+  return e == cudaSuccess ? launch_publish(h, st) : e;
+}
+
+// The same as a CUDA graph (use_graphs; the arguments are the handle's buffers):
+// some 30 dependent launches of a few microseconds, which the host issues more
+// slowly than a small system runs them (30 buses x 24 periods: a solve 195 us
+// directly, 137 us so; factor and solve 530 and 465 us).  On any failure the
+// handle launches them directly from then on.
+void build_apply_graph(Handle& h, bool refine) {
+  const int sf = h.s_factor, kind = refine ? 1 : 0;
+  cudaGraphExec_t& exec = h.app_exec[sf][kind];
+  const int64_t l0 = h.launches;
+  cudaGraph_t g = nullptr;
+  cudaError_t e = cudaStreamBeginCapture(h.cap_stream, cudaStreamCaptureModeThreadLocal);
+  if (e == cudaSuccess) {
+    const cudaError_t e1 = enqueue_apply(h, refine, h.cap_stream);
+    const cudaError_t e2 = cudaStreamEndCapture(h.cap_stream, &g);
+    e = e1 != cudaSuccess ? e1 : e2;
+  }
+  if (e == cudaSuccess && g) e = cudaGraphInstantiate(&exec, g, 0);
+  if (g) cudaGraphDestroy(g);
+  h.app_launches[sf][kind] = h.launches - l0;
+  h.launches = l0;
+  if (e != cudaSuccess || !exec) {
+    exec = nullptr;
+    h.app_seen[sf][kind] = -1;
+    (void)cudaGetLastError();
+  }
+}
+
+// When a graph is built (some 100 us of the host's time for 30 launches): that of
+// the first application at the end of the handle's first kkt_factor, while the
+// device is busy with the factor; the others at their second use, so that a
+// solve with one refinement step, and a fallback, pay for none.  The first,
+// second and later solves of a handle on 30 buses x 24 periods: 185, 151 and 142
+// us (227, 261 and 142 with every graph built at its second use, 249, 226 and 224
+// with no graphs and the norms copied back); 301 x 48 332, 283 and 277 (396, 418
+// and 277; 646, 610 and 607).  The first factor takes as long as before (0.51 and
+// 1.92 ms).
+cudaError_t run_apply(Handle& h, bool refine, cudaStream_t st) {
+  const int sf = h.s_factor, kind = refine ? 1 : 0;
+  cudaGraphExec_t& exec = h.app_exec[sf][kind];
+  if (!exec && h.opt.use_graphs && h.app_seen[sf][kind] >= 0 && h.app_seen[sf][kind]++ > 0) build_apply_graph(h, refine);
+  if (!exec) return enqueue_apply(h, refine, st);
+  h.launches += h.app_launches[sf][kind];
+  return cudaGraphLaunch(exec, st);
+}
+
 // The factor of the input values with the inertia-correction shift (dw, dc;
 // dcs on C's diagonal) applied to the device copy (none when dw and dc are 0).
 kkt_status factor_values(Handle* h, const double* a_vals, const double* b_vals, const double* c_vals,
@@ -1007,6 +1063,10 @@ kkt_status factor_values(Handle* h, const double* a_vals, const double* b_vals, 
   h->front_done = false;
   h->factored = with_s;
   h->timed_factor = with_s;
+  if (with_s && h->factor_exec && !h->opt.early_solve && !h->opt.device_refine && h->app_seen[h->s_factor][0] == 0) {
+    h->app_seen[h->s_factor][0] = 1;
+    build_apply_graph(*h, false);
+  }
   return KKT_OK;
 }
 
@@ -1098,52 +1158,6 @@ void build_solve_graph(Handle& h) {
     h.solve_exec[sf] = nullptr;
     (void)cudaGetLastError();
   }
-}
-
-// kkt_solve's host loop up to its next look at the norms: the application of
-// the factorization to h.rhs into h.x, or with `refine` to the residual and x +=
-// dx; then the residual, its norms and what the test reads.
-cudaError_t enqueue_apply(Handle& h, bool refine, cudaStream_t st) {
-  cudaError_t e = refine ? launch_apply_inverse(h, h.rho, h.dx, st) : launch_apply_inverse(h, h.rhs, h.x, st);
-  if (e == cudaSuccess && refine) e = launch_axpy(h, h.x, h.dx, (int64_t)h.N * h.nA + h.nC, st);
-  if (e == cudaSuccess) e = launch_residual(h, h.rhs, h.x, h.rho, st);
-  if (e == cudaSuccess) e = launch_norms(h, h.rho, h.x, h.rhs, st);
-  return e == cudaSuccess ? launch_publish(h, st) : e;
-}
-
-// The same as a CUDA graph from the handle's second such call on (use_graphs;
-// the arguments are the handle's buffers): some 30 dependent launches of a few
-// microseconds, which the host issues more slowly than a small system runs them
-// (30 buses x 24 periods: a solve 195 us directly, 137 us so; factor and solve
-// 530 and 465 us).
-// A handle that solves once does not pay for the capture.
-cudaError_t run_apply(Handle& h, bool refine, cudaStream_t st) {
-  const int sf = h.s_factor, kind = refine ? 1 : 0;
-  if (!h.opt.use_graphs || h.app_seen[sf][kind] < 0 || h.app_seen[sf][kind]++ == 0) return enqueue_apply(h, refine, st);
-  cudaGraphExec_t& exec = h.app_exec[sf][kind];
-  if (!exec) {
-    const int64_t l0 = h.launches;
-    cudaGraph_t g = nullptr;
-    cudaError_t e = cudaStreamBeginCapture(h.cap_stream, cudaStreamCaptureModeThreadLocal);
-    if (e == cudaSuccess) {
-      const cudaError_t e1 = enqueue_apply(h, refine, h.cap_stream);
-      const cudaError_t e2 = cudaStreamEndCapture(h.cap_stream, &g);
-      e = e1 != cudaSuccess ? e1 : e2;
-    }
-    if (e == cudaSuccess && g) e = cudaGraphInstantiate(&exec, g, 0);
-    if (g) cudaGraphDestroy(g);
-    h.app_launches[sf][kind] = h.launches - l0;
-    h.launches = l0;
-    if (e != cudaSuccess || !exec) {
-      exec = nullptr;
-      h.app_seen[sf][kind] = -1;  // launch directly from now on
-      (void)cudaGetLastError();
-      return enqueue_apply(h, refine, st);
-    }
-  }
-  h.app_seen[sf][kind] = 1;
-  h.launches += h.app_launches[sf][kind];
-  return cudaGraphLaunch(exec, st);
 }
 
 // One cycle of GMRES refinement (right preconditioning by the factorization

@@ -276,7 +276,8 @@ struct Handle {
   bool solve_graph_failed[2] = {false, false};
   double* rstate = nullptr;
   // graphs of kkt_solve's host loop, per kind of factor of S: [0] the first
-  // application with its residual and norms, [1] one refinement step with them
+  // application with its residual and norms, [1] one refinement step with them;
+  // app_seen: uses so far while there is no graph, -1 if it could not be built
   cudaGraphExec_t app_exec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
   int64_t app_launches[2][2] = {{0, 0}, {0, 0}};
   int app_seen[2][2] = {{0, 0}, {0, 0}};

@@ -141,8 +141,11 @@ typedef struct {
                            (mode 1) or 96 GiB (mode 2).  The same static-pivot rule applies; the
                            factor is scattered back into the supernodal panels.
                            0: off; 1: trailing updates in FP64 on the CUDA cores; 2: trailing
-                           updates in emulated FP64 on the tensor cores (7 base-256 digit
-                           slices per operand, as in KKT_F64_EMULATED); -1 (default): 2 in the
+                           updates and, with at least 512 columns, the panels and the updates by
+                           descendants outside the tail with many rows in it, in emulated FP64
+                           on the tensor cores (7 base-256 digit slices per operand, as in
+                           KKT_F64_EMULATED: 55 bits relative to the largest entry of a row over
+                           up to 256 columns); -1 (default): 2 in the
                            KKT_TF32, KKT_BF16 and KKT_F64_EMULATED modes, 1 in KKT_FP64 (all its
                            arithmetic stays FP64 on the CUDA cores). */
   int32_t autotune;     /* choose the size of the dense tail by timing: the tail is the longest suffix
@@ -548,10 +551,10 @@ kkt_status kkt_kernel_stats(kkt_handle* h, int32_t family, kkt_kernel_stat* out)
 kkt_status kkt_measure_fp64_peak(double* gflops);
 
 /* Diagnostic: for n device doubles d, recip[i] = the reciprocal the factor
- * kernels take of a pivot d[i] (an FP32 seed and two FP64 Newton-Raphson
- * steps; CUDA's division for |d| outside [1e-36, 1e36]) and quotient[i] =
- * 1.0 / d[i] by CUDA's FP64 division, so that tests can bound the
- * difference.  Device arrays; asynchronous on `stream`. */
+ * kernels take of a pivot d[i] (an FP32 seed and a three-term series in
+ * integer arithmetic; CUDA's division for |d| outside [2^-119, 2^120)) and
+ * quotient[i] = 1.0 / d[i] by CUDA's FP64 division, so that tests can bound
+ * the difference.  Device arrays; asynchronous on `stream`. */
 kkt_status kkt_probe_pivot_reciprocal(const double* d, int64_t n, double* recip, double* quotient, void* stream);
 
 /* Diagnostic: leaves the handle as a bounded device wait that runs out on

@@ -58,13 +58,17 @@ kkt_status cuda_status(cudaError_t e, const char* what) {
 void free_all(Handle* h) {
   void* ptrs[] = {h->d.sn_first, h->d.sn_rowptr, h->d.sn_rows, h->d.sn_valoff, h->d.upd_ptr,
                   h->d.upd_src, h->d.upd_r0, h->d.upd_r1, h->d.upd_reloff, h->d.upd_rel,
-                  h->d.lvl_sn, h->d.perm, h->d.a_map, h->d.col_primal, h->d.col_dpos, h->d.diag_pos, h->d.fwork, h->d.fpairs,
+                  h->d.lvl_sn, h->d.perm, h->d.a_map, h->d.col_primal, h->d.col_dpos, h->d.diag_pos, h->d.fwork,
+                  h->d.fpairs,
                   h->d.full_rowptr, h->d.full_col, h->d.full_src, h->d.b_row, h->d.b_col,
                   h->d.b_blockptr, h->d.e_t, h->d.e_block, h->d.wpos, h->d.sn_wrow, h->d.w_dpos,
                   h->d.w_col, h->d.reach_lvl_sn, h->d.s_key, h->d.s_ptr, h->d.s_e1, h->d.s_e2,
                   h->d.t_ptr, h->d.t_e, h->d.bt_ptr, h->d.E, h->d.g_rows, h->d.trsv_jlo, h->d.trsv_jhi,
-                  h->d.panel_small, h->d.panel_items, h->d.flvl_desc, h->d.fr_ptr, h->d.fr_rec, h->d.wr_ptr, h->d.wr_row, h->d.w_sn, h->d.twork, h->d.tpairs, h->d.upd_ntail, h->d.reach_lvl_sn_nt, h->d.tail_sn_list, h->d.hv_off, h->d.hv_sn, h->d.hv_col, h->d.hv_pos, h->d.tail_wrow, h->d.wt_ptr, h->d.wt_idx,
-                  h->d.g_key, h->d.g_ptr, h->d.g_row, h->Xinv, h->Sdinv, h->wdinv, h->Xtail, h->Tt, h->TY, h->t_imgA, h->t_imgB,
+                  h->d.panel_small, h->d.panel_items, h->d.flvl_desc, h->d.fr_ptr, h->d.fr_rec, h->d.wr_ptr,
+                  h->d.wr_row, h->d.w_sn, h->d.twork, h->d.tpairs, h->d.upd_ntail, h->d.reach_lvl_sn_nt,
+                  h->d.tail_sn_list, h->d.hv_off, h->d.hv_sn, h->d.hv_col, h->d.hv_pos, h->d.tail_wrow, h->d.wt_ptr,
+                  h->d.wt_idx, h->d.g_key, h->d.g_ptr, h->d.g_row, h->Xinv, h->Sdinv, h->wdinv, h->Xtail, h->Tt, h->TY,
+                  h->t_imgA, h->t_imgB,
                   h->t_scaleA, h->t_scaleB, h->Lx, h->LDx, h->a_vals, h->b_vals,
                   h->c_vals, h->anorm, h->W, h->G, h->S, h->Ypanel, h->knorm, h->counters, h->r,
                   h->z, h->u, h->v, h->tg, h->xg, h->x, h->dx, h->rho, h->rhs, h->red,
@@ -414,8 +418,9 @@ kkt_status analyze_one(const kkt_pattern* pat, const kkt_options* opt, double ta
   h->hv_cols = (int32_t)hv_off.size();
 
   // factor work items: 32-row tiles of every supernode outside the dense tail,
-  // grouped by level; per item the updates that meet the tile, as (update index within s's list, rows [ia, ib) of the
-  // descendant that land in the tile), from the item's offset to the next item's
+  // grouped by level; per item the updates that meet the tile, as (update index
+  // within s's list, rows [ia, ib) of the descendant that land in the tile), from
+  // the item's offset to the next item's
   std::vector<int32_t> fwork, twork, flvl_sn;
   std::vector<TailPair> tpairs;
   std::vector<UpdPair> fpairs;

@@ -1102,8 +1102,9 @@ __device__ __forceinline__ void slice_columns(const double (&v)[kEwWarpCols], in
 // rows rho in [0, mpad) of the outer trailing matrix of matrix blockIdx.y:
 // operand A = rows of Y (columns 0..kw-1 of Yw, leading dimension n), operand
 // B = rows of L (columns K0..K0+kw-1 of S); rows >= m and columns >= kw are zero.
-// 32 rows of one operand per CTA: lane l takes row l, warp w the columns 32 w .., read once, all loads in flight together, and kept in registers
-// while the row's scale is found.  One matrix of order 1,848: 8.4 us (106 with a
+// 32 rows of one operand per CTA: lane l takes row l, warp w the columns 32 w ..,
+// read once, all loads in flight together, and kept in registers while the row's
+// scale is found.  One matrix of order 1,848: 8.4 us (106 with a
 // thread per row that read its 256 columns twice), 24 of order 7,000: 108 us
 // (281).
 __global__ void __launch_bounds__(256, 2) k_slice_wide(const double* __restrict__ S0, const double* __restrict__ Yw0,
@@ -1141,9 +1142,10 @@ __global__ void __launch_bounds__(256, 2) k_slice_wide(const double* __restrict_
 // panels of the heavy descendants: B = L, A = L D over their columns, rows = the
 // tail's nT rows (zero where a descendant has none).  A column with pivot d is
 // balanced by an exact power of two, L 2^h and L D 2^-h with 2^(2h) about |d|:
-// the row scales then follow |L_ik| |d_k|^(1/2), whose squares the diagonal
-// entries of the matrix bound, instead of the spread of the pivots.  32 rows of
-// one operand per CTA, as k_slice_wide.
+// the row scales then follow max_k |L_ik| |d_k|^(1/2) instead of the spread of the
+// pivots, and the product's error is relative to the product of two such scales,
+// that is to the growth |L||D||L|^T.  (The pivots have both signs, so the diagonal
+// of the matrix does not bound it.)  32 rows of one operand per CTA, as k_slice_wide.
 __global__ void __launch_bounds__(256, 2) k_slice_heavy(const double* __restrict__ Lx, int64_t pt,
                                                      const double* __restrict__ LDx, int64_t ldt,
                                                      const int64_t* __restrict__ off, const int32_t* __restrict__ sn,

@@ -116,9 +116,6 @@ KKT_HD void balanced7(unsigned long long q, int (&d)[kEmuSlices]) {
   }
 }
 
-// Biased exponent field of a double (0 for zero and subnormals).
-KKT_HD int exp_field(double v) { return (int)((bits_of(v) >> 52) & 0x7FF); }
-
 // Bits of |v|: as unsigned integers they order like the magnitudes, so a row's
 // largest one is found without the FP64 pipe.
 KKT_HD unsigned long long magnitude_bits(double v) { return (unsigned long long)bits_of(v) & 0x7FFFFFFFFFFFFFFFull; }

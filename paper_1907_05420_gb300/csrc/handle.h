@@ -52,6 +52,9 @@ constexpr int kTailTileRows = 4;
 // Columns of a tile: wide tiles meet a descendant less often, narrow ones spread
 // a small tail over more warps.  48 tails of order 130: 60 us with 64 columns, 92
 // with 128; 96 of order 724: 1.55 and 1.50 ms; 24 of order 6,938: 16.5 and 13.4 ms.
+// Whole block factors, 64 and 128: order 198 1.453 and 1.473 ms, 310 1.392 and 1.423,
+// 376 2.022 and 2.028, 552 3.844 and 3.876, 704 22.65 and 22.65, 899 11.17 and 11.16,
+// 7,092 55.04 and 54.02: even from 550 to 900, where the line lies.
 inline int tail_tile_cols(int nT) { return nT >= 512 ? 128 : 64; }
 
 // One entry of a row's list for the forward solve: the row's entries in the panel
@@ -71,7 +74,9 @@ static_assert(sizeof(SnDesc) == 32, "SnDesc layout");
 // The block factor's panels: eight lanes take a panel of at most kPanelSmall
 // entries; a larger one has an item for its triangle and its rows or, with more
 // than kPanelRows rows below the triangle, for the triangle alone and one per
-// kPanelTile rows.  kPanelSmall: 16 panels stay within 16.5 KB per CTA.
+// kPanelTile rows.  kPanelSmall: 16 panels stay within 16.5 KB per CTA; 64 entries
+// make the block factor 0.2 to 6% slower.  kPanelRows of 128 or 512 and kPanelTile of
+// 64 or 256 change it by 0.3% at most (118 to 9,241 buses).
 constexpr int kPanelSmall = 128, kPanelRows = 256, kPanelTile = 128;
 struct alignas(16) PanelItem {
   int64_t val;                  // offset of the panel
@@ -82,7 +87,10 @@ static_assert(sizeof(PanelItem) == 32, "PanelItem layout");
 struct PanelLevel {
   int32_t small0 = 0, nsmall = 0, item0 = 0, nitems = 0, nrows = 0;  // items: nitems, then nrows for the second launch
 };
-// Supernodes that eight lanes solve with (at most this many columns and rows).
+// Supernodes that eight lanes solve with (at most this many columns and rows).  A
+// solve with 24, 48, 96 rows and with none: 301 buses x 48 periods 244, 276, 281 and
+// 308 us, 500 x 96 456, 486, 510 and 723, 2,383 x 96 1.80, 1.80, 1.83 and 3.21 ms,
+// 9,241 x 8 2.59, 2.55, 2.60 and 2.99; with four columns 2 to 17% more than with eight.
 constexpr int kSmallSnCols = 8, kSmallSnRows = 48;
 
 // Device copies of the symbolic structures.
@@ -140,7 +148,7 @@ struct DevSym {
   int32_t* wr_ptr = nullptr;       // per column of W: its nonzero rows outside the (augmented) tail
   int32_t* wr_row = nullptr;
   int32_t* w_sn = nullptr;         // per W row: its supernode
-  int32_t* twork = nullptr;        // tiles of the dense tail with updates from outside: 3 ints, tile row, tile column, first pair
+  int32_t* twork = nullptr;        // tiles of the dense tail with updates from outside: tile row, tile column, first pair
   TailPair* tpairs = nullptr;
   int32_t* upd_ntail = nullptr;    // per supernode: leading updates from outside the tail
   int32_t* reach_lvl_sn_nt = nullptr;  // reach supernodes outside the tail, by level
@@ -248,7 +256,7 @@ struct Handle {
   bool g_reduced = false;     // S assembled from a TF32/BF16 contraction
   int g_nchunks = 0, g_nchunks_pos = 0;  // 64-row chunks of g_rows (positive-pivot chunks first)
   double* knorm = nullptr;    // ||K||_inf
-  unsigned long long* counters = nullptr;  // 2 kNumCounters; dev_err behind them, cleared with them by every factor
+  unsigned long long* counters = nullptr;  // 2 kNumCounters and dev_err, cleared together by every factor
   // solve work vectors
   double* r = nullptr;        // nK: right-hand side being solved
   double* z = nullptr;        // N * nA

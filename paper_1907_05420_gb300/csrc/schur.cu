@@ -249,9 +249,12 @@ __global__ void __launch_bounds__(256) k_assemble_s_warp(
   }
 }
 
-// Records per entry of S from which a warp takes an entry.  SCOPF with 16
-// outages on 1,021 buses, 862 records per entry: 0.91 ms with a warp, 18.9 with a
-// thread; the adjacent coupling has one to four.
+// Records per entry of S from which a warp takes an entry.  Whole assembly, thread
+// and warp: the adjacent coupling (1.3 records) on 301 buses x 48 periods 32 and 43
+// us, on 2,383 x 96 0.48 and 1.87 ms; the cumulative coupling on 200 buses with 5
+// records 26 and 24 us, 12.8 45 and 33, 23 61 and 43, 66 176 and 167; SCOPF on 60
+// buses with 79 164 and 25, on 1,021 buses (862) 18.9 and 0.91 ms.  They cross
+// between 1.3 and 5, where the two differ by few microseconds on systems this small.
 constexpr int64_t kAssembleWarpRecords = 16;
 
 }  // namespace

@@ -626,7 +626,10 @@ __global__ void k_scale_into(double* __restrict__ y, double a, const double* __r
 // Lanes per coupling column: a warp from 16 entries per column on, and for a
 // dense C (a row of nC entries).  1,021 buses with 16 outages (304 columns of some
 // 121 entries): t 13 us (214 with a thread per column), the residual's coupling
-// rows 14 (204), their norm 9 (101).
+// rows 14 (204), their norm 9 (101).  A solve of the cumulative coupling on 200
+// buses, a thread and a warp per column: 211 and 207 us with 9 entries, 231 and 218
+// with 17, 331 and 289 with 49; with the two of the adjacent coupling the same to
+// 0.5%, where a thread keeps the launches small.
 inline int coupling_lanes(const Handle& h) { return h.c_kind == 1 || h.nnzB >= 16 * (int64_t)h.nC ? 32 : 1; }
 inline int coupling_grid(const Handle& h) { return (int)(((int64_t)h.nC * coupling_lanes(h) + 255) / 256); }
 
@@ -681,7 +684,8 @@ cudaError_t launch_apply_front(Handle& h, const double* r, cudaStream_t st) {
     if (k > 0 && nw > 0) {
       dim3 g((k + 31) / 32, N);
       {
-    k_reduce_u<<<g, 32 * kReduceWarps, 0, st>>>(h.W, h.z, h.wdinv, h.d.w_col, h.d.wr_ptr, h.d.wr_row, h.nw_nt, nw, k, nA, h.u);
+    k_reduce_u<<<g, 32 * kReduceWarps, 0, st>>>(h.W, h.z, h.wdinv, h.d.w_col, h.d.wr_ptr, h.d.wr_row, h.nw_nt, nw, k,
+                                                nA, h.u);
     h.launches++;
   }
     } else if (k > 0) {
@@ -714,8 +718,8 @@ cudaError_t launch_apply_back(Handle& h, double* out, cudaStream_t st, bool solv
     h.launches++;
   }
       {
-    k_apply_xg<<<(int)(((int64_t)nw * N * 8 + 255) / 256), 256, 0, st>>>(h.W, h.v, h.d.w_col, h.d.w_sn, h.d.wt_ptr, h.d.wt_idx,
-                                                          h.nw_nt, nw, k, nA, N, h.z);
+    k_apply_xg<<<(int)(((int64_t)nw * N * 8 + 255) / 256), 256, 0, st>>>(
+        h.W, h.v, h.d.w_col, h.d.w_sn, h.d.wt_ptr, h.d.wt_idx, h.nw_nt, nw, k, nA, N, h.z);
     h.launches++;
   }
     }
@@ -866,7 +870,8 @@ cudaError_t launch_apply_inverse_ws(Handle& h, const double* r, double* out,
   if (h.nC > 0) {
     if (k > 0 && nw > 0) {
       dim3 g((k + 31) / 32, N);
-      k_reduce_u<<<g, 32 * kReduceWarps, 0, st>>>(h.W, ws.z, h.wdinv, h.d.w_col, h.d.wr_ptr, h.d.wr_row, h.nw_nt, nw, k, nA, ws.u);
+      k_reduce_u<<<g, 32 * kReduceWarps, 0, st>>>(h.W, ws.z, h.wdinv, h.d.w_col, h.d.wr_ptr, h.d.wr_row, h.nw_nt, nw,
+                                                  k, nA, ws.u);
       h.launches++;
     } else if (k > 0) {
       cudaError_t e = cudaMemsetAsync(ws.u, 0, sizeof(double) * (size_t)k * N, st);
@@ -879,8 +884,8 @@ cudaError_t launch_apply_inverse_ws(Handle& h, const double* r, double* out,
     if (e != cudaSuccess) return e;
     if (k > 0 && nw > 0) {
       k_mx<<<(k * N + 255) / 256, 256, 0, st>>>(h.d.bt_ptr, h.d.b_col, h.b_vals, ws.xg, k, N, ws.v);
-      k_apply_xg<<<(int)(((int64_t)nw * N * 8 + 255) / 256), 256, 0, st>>>(h.W, ws.v, h.d.w_col, h.d.w_sn, h.d.wt_ptr, h.d.wt_idx,
-                                                            h.nw_nt, nw, k, nA, N, ws.z);
+      k_apply_xg<<<(int)(((int64_t)nw * N * 8 + 255) / 256), 256, 0, st>>>(
+          h.W, ws.v, h.d.w_col, h.d.w_sn, h.d.wt_ptr, h.d.wt_idx, h.nw_nt, nw, k, nA, N, ws.z);
       h.launches += 2;
     }
   }

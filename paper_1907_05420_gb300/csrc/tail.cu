@@ -11,11 +11,11 @@
 // Per factor: the tail panels (A's values) are gathered into the zeroed dense
 // triangles, which then take the updates from outside the tail; each 64-wide
 // panel step factors the diagonal blocks of all N triangles (with the
-// static-pivot rule and the inertia counts of the sparse panels), forms L21 and Y = L21 D, and updates the trailing triangles, in
-// FP64 on the CUDA cores (tail mode 1) or in emulated FP64 on the tensor cores
-// (tail mode 2, the update of dense_tc.cu: 7 base-256 digit slices per
-// operand); the factor is scattered back into the supernodal panels, which
-// the solves use.
+// static-pivot rule and the inertia counts of the sparse panels), forms L21 and
+// Y = L21 D, and updates the trailing triangles, in FP64 on the CUDA cores (tail
+// mode 1) or in emulated FP64 on the tensor cores (tail mode 2, the update of
+// dense_tc.cu: 7 base-256 digit slices per operand); the factor is scattered back
+// into the supernodal panels, which the solves use.
 // Entries of the triangles outside the supernodal structure stay exact zeros
 // (every product that reaches them has a zero factor).
 //

@@ -83,8 +83,8 @@ __global__ void k_tail_aug_rows(double* __restrict__ W, int nw, int k, double* _
 // warp on its own: no barrier between descendants) and subtracts it from the
 // dense triangle at the end.
 // What bounds it: latency, about two round trips to L2 per descendant and tile,
-// hidden by 40 warps per SM with small tiles; then the FP64 pipe, which the few
-// entries of a descendant in a tile fill by a third.  The CTA-wide staging of
+// hidden by 40 warps per SM with small tiles; then the FP64 pipe, 72% busy on 24
+// tails of order 732 and 68% on 8 of order 7,009, where L1 is at 78%.  The CTA-wide staging of
 // k_factor_update, with two barriers per descendant, took 138 us for 48 tails of
 // order 130 (60 here), 2.8 ms for 96 of order 724 (1.5) and, without their heavy
 // descendants, 56 ms for 24 of order 6,938 (13.4); loading the next descendant
